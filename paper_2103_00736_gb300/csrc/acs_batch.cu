@@ -245,7 +245,7 @@ void layout(Batch* B, Pool& P) {
     B->d_head = P.take<int>(32);
     B->d_mailbox = P.take<int>(B->max_ctas);
     B->d_team_bar = P.take<unsigned long long>(B->max_ctas);
-    B->d_team_part = P.take<double>((size_t)B->max_ctas * kMaxRed);
+    B->d_team_part = P.take<double>((size_t)B->max_ctas * kPartStride);
     B->d_team_err = P.take<int>(B->max_ctas);
     B->d_dense = P.take<double>(B->dense_m2 > 0 ? (size_t)B->max_ctas * 2 * B->dense_m2 : 1);
     B->total_bytes = P.off;

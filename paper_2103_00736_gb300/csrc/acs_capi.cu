@@ -556,7 +556,7 @@ int acs_problem_create(int32_t m, int32_t n, const int64_t* row_ptr, const int32
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, P->device);
     P->max_ctas = (nsm > 0 ? nsm : 1) * 8;
-    if (dalloc(P, &P->partials, (size_t)P->max_ctas * acs::kMaxRed) || dalloc(P, &P->flags, P->max_ctas) ||
+    if (dalloc(P, &P->partials, (size_t)P->max_ctas * acs::kPartStride) || dalloc(P, &P->flags, P->max_ctas) ||
         dalloc(P, &P->release, 32) || dalloc(P, &P->bcast, acs::kMaxRed) ||
         dalloc(P, &P->ctl, 1)) { free_all(P); delete P; return ACS_ERR_OOM; }
     if (cudaMallocHost(&P->ctl_host, sizeof(acs::Control)) != cudaSuccess) { free_all(P); delete P; return ACS_ERR_OOM; }

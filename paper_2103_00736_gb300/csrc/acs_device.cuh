@@ -33,33 +33,64 @@ __device__ __forceinline__ int ld_volatile_int(const int* p) { return *(volatile
 
 // Grid-wide reduction and barrier.
 //
-// A phase leaves its contributions to a reduction in shared memory
-// (block_partials: warp shuffles, then one warp combines the warps in fixed
-// order).  grid_sync then publishes this CTA's partials followed by an
-// arrival flag holding the barrier generation; thread b of every CTA waits
-// for the flag of CTA b and loads CTA b's partials, and the CTA combines them
-// in CTA order (a fixed shuffle tree, then the warps in order).  Every CTA
-// thus computes bit-identical reduced values (deterministic for a given
-// launch shape) after a single one-way flag latency.  All waits are bounded
+// A phase leaves its contributions to a reduction in shared memory as one
+// value per warp (block_partials).  At the barrier that ends the phase warp 0
+// combines the warps and publishes this CTA's partials, the first warps read
+// every CTA's partials and combine them in a fixed order, and warp 0 alone
+// computes the scalars that steer the loop from them (the `post` function of
+// grid_sync_post); everyone else waits at the CTA barrier that follows and
+// reads the results in shared memory.  Every CTA thus holds bit-identical
+// values (deterministic for a given launch shape).  What bounds these steps
+// is the FP64 pipe: it takes a warp instruction in 16 cycles per SM, so a
+// scalar operation repeated by all 32 warps costs 512 cycles, and a dependent
+// addition has a latency of 64, so a chain of square root and quotients takes
+// about 1 us even in one warp.  Measured on 152 CTAs: a barrier that reduces
+// one value 5.2 -> 3.9 us, the CG vector step of a 2000-row dense problem
+// 13.7 -> 8.7 us, a KKT check of a 1000 x 5000 LP 34 -> 21 us (before: every
+// CTA read the partials after the counter had arrived, and every thread
+// computed the scalars).
+// All waits are bounded
 // (kBarrierTimeoutNs): on expiry, or when another CTA has recorded an error,
 // the wait records ACS_ERR_DEVICE_TIMEOUT and grid_sync returns false in
 // every thread; the caller then leaves the kernel.
 constexpr int kMaxGrid = 256;   // CTAs of a persistent launch (one per SM)
 
+// Scalars that steer the solve loop and the CG, computed once per CTA.
+struct CondRange {
+    double alpha, lmin, lmax;
+    bool any;
+};
+struct LoopScalars {
+    double gam, gam_prev, alpha, alpha_prev, beta, thr;   // CG
+    double floor_r, target, best, best_ref;               // polish solves
+    double ds, snorm, eta, d0, d1;                        // step norms, inexactness factor
+    double res[6], best_mx;                               // residuals of the last check
+    CondRange range;                                      // exponent range of a rescaling
+    int flat_checks;
+    int go;          // CG: the residual is above its target
+    int far;         // CG: ... by more than a factor 100
+    int bad;         // a non-finite value
+    int broke;       // CG: p'Mp <= 0
+    int over;        // the deadline of a time-sliced solve has passed
+    int trouble;     // the FP32 correction cannot keep up
+    int solved;      // every residual is <= tol
+    int end32;       // the FP32 outer passes end
+};
+
 struct SyncShared {
     int team_rank;            // this CTA's rank in the team working on one problem
     int team_size;            // CTAs in the team (the whole grid for a single solve)
     unsigned long long* bar;  // the team's monotonic barrier arrival counter
-    double* tpart;            // the team's partials, [team_size * kMaxRed]
+    double* tpart;            // the team's partials, [team_size * kPartStride]
     double* dM;               // the team's dense scratch for the cached projection operator:
     double* dX;               //   M / its Cholesky factor and L^{-1}, [m * m] each
     unsigned long long deadline;  // global-timer time at which a time-sliced solve pauses (0 = none)
-    double blk[kMaxRed];      // this CTA's partials
     double out[kMaxRed];      // grid-reduced values of the last barrier
-    double wsum[kWarps][kMaxRed];
-    double gath[kMaxRed][kMaxGrid];   // every CTA's partials, gathered
-    int op[kMaxRed];          // 0 = sum, 1 = max
+    double wsum[kWarps][kMaxRed];   // the warps' contributions to the next one
+    double gsum[kWarps][kMaxRed];   // the CTAs' contributions, by the warp that gathered them
+    unsigned opmask;          // bit k: value k is combined by max (else by sum)
     int nv;                   // number of values reduced at the next barrier
+    LoopScalars lp;           // scalars of the solve loop, written by warp 0 at the barriers
     int fail;
     unsigned gen;             // barrier generation (same sequence in every CTA)
     // column-blocked passes: the mbarrier that completes a block's bulk copy
@@ -112,29 +143,98 @@ __device__ __forceinline__ double warp_max(double x) {
     return x;
 }
 
-// Stage this CTA's contribution to the values reduced at the next grid_sync.
+// Sums over the warp of NV values at once: at each of the first steps a lane
+// gives half of its values to its partner and keeps the other half, so that 8
+// values take 9 FP64 additions a lane instead of 40.  On return v[0] of lane l
+// holds value warp_sums_index<NV>(l), for l a multiple of 32 / NV.
 template <int NV>
-__device__ void block_partials(const double (&v)[NV], const int (&op)[NV], double* /*unused*/) {
+__device__ __forceinline__ void warp_sums(double (&v)[NV]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int c = NV; c > 1; c >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < c / 2; ++i) {
+            const double give = up ? v[i] : v[i + c / 2];
+            const double keep = up ? v[i + c / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+template <int NV>
+__device__ __forceinline__ int warp_sums_index(int lane) {
+    return NV == 1 ? 0 : NV == 2 ? lane >> 4 : NV == 4 ? lane >> 3 : lane >> 2;
+}
+
+__device__ __forceinline__ bool is_nonzero(double x) {   // without the FP64 pipe
+    return (__double_as_longlong(x) << 1) != 0ll;
+}
+
+// Stage this CTA's contribution to the values reduced at the next grid_sync:
+// one value per warp (warps with nothing but zeros skip their sums).  op: 0 =
+// sum, 1 = max.
+template <int NV>
+__device__ __forceinline__ void block_partials(const double (&v)[NV], const int (&op)[NV], double* /*unused*/) {
     SyncShared& S = sync_smem();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned mask = 0u;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const double x = op[k] ? warp_max(v[k]) : warp_sum(v[k]);
-        if (lane == 0) S.wsum[warp][k] = x;
-    }
-    __syncthreads();
-    if (warp == 0) {
+    for (int k = 0; k < NV; ++k) mask |= (op[k] ? 1u : 0u) << k;
+    if (mask == 0u) {
+        constexpr int NP = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : 8;
+        double a[NP];
+        bool nz = false;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            a[k] = k < NV ? v[k < NV ? k : 0] : 0.0;
+            nz |= is_nonzero(a[k]);
+        }
+        if (__any_sync(0xffffffffu, nz)) warp_sums<NP>(a);
+        else a[0] = 0.0;
+        const int k = warp_sums_index<NP>(lane);
+        if ((lane & (32 / NP - 1)) == 0 && k < NV) S.wsum[warp][k] = a[0];
+    } else {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            double x = (lane < (int)(blockDim.x >> 5)) ? S.wsum[lane][k] : (op[k] ? -INFINITY : 0.0);
-            x = op[k] ? warp_max(x) : warp_sum(x);
-            if (lane == 0) {
-                S.blk[k] = x;
-                S.op[k] = op[k];
-            }
+            const double x = op[k] ? warp_max(v[k]) : warp_sum(v[k]);
+            if (lane == 0) S.wsum[warp][k] = x;
         }
-        if (lane == 0) S.nv = NV;
     }
+    if (threadIdx.x == 0) {
+        S.opmask = mask;
+        S.nv = NV;
+    }
+}
+
+// Combine over the warp's lanes the nv values each lane holds, into dst[0, nv).
+template <int NV>
+__device__ __forceinline__ void warp_sums_to(const double (&x)[kMaxRed], int nv, double* dst) {
+    const int lane = threadIdx.x & 31;
+    double a[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) a[k] = x[k];
+    warp_sums<NV>(a);
+    const int k = warp_sums_index<NV>(lane);
+    if ((lane & (32 / NV - 1)) == 0 && k < nv) dst[k] = a[0];
+}
+__device__ __forceinline__ void warp_combine(const double (&x)[kMaxRed], int nv, unsigned opmask, double* dst) {
+    if (opmask == 0u) {
+        if (nv <= 1) warp_sums_to<1>(x, nv, dst);
+        else if (nv <= 2) warp_sums_to<2>(x, nv, dst);
+        else if (nv <= 4) warp_sums_to<4>(x, nv, dst);
+        else warp_sums_to<8>(x, nv, dst);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kMaxRed; ++k)
+            if (k < nv) {
+                const double r = (opmask >> k) & 1u ? warp_max(x[k]) : warp_sum(x[k]);
+                if ((threadIdx.x & 31) == 0) dst[k] = r;
+            }
+    }
+    __syncwarp();
 }
 
 // Start (or resume, with the generation reached so far) the team's barrier
@@ -158,88 +258,173 @@ __device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long l
     return v;
 }
 
-// Barrier: thread 0 of every CTA of the team publishes the CTA's partials,
-// adds 1 to the team's monotonic arrival counter with release semantics and
-// spins (acquire) until the counter reaches (generation) * (CTAs in the team).
-// A team of one CTA needs no counter: its partials are already combined.  One thread per CTA polls a
-// single word, which keeps the barrier at about the latency of two L2 round
-// trips.  The partials of all CTAs are then read once, in parallel.
-static __device__ __noinline__ bool grid_sync(int* err) {
+// A partial and the generation of the barrier it belongs to, written and read
+// as one 16-byte access: a reader that sees the generation has the value.
+__device__ __forceinline__ void st_slot(double* slot, double v, unsigned long long tag) {
+    asm volatile(
+        "{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(slot),
+        "l"(__double_as_longlong(v)), "l"(tag)
+        : "memory");
+}
+__device__ __forceinline__ double ld_slot(const double* slot, unsigned long long& tag) {
+    long long v;
+    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
+                 : "=l"(v), "=l"(tag)
+                 : "l"(slot)
+                 : "memory");
+    return __longlong_as_double(v);
+}
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// A bounded wait's bookkeeping: called with the number of unsuccessful tries
+// so far; true when the wait must end (another CTA recorded an error, or the
+// time is up, which records ACS_ERR_DEVICE_TIMEOUT).
+__device__ __forceinline__ bool wait_expired(int tries, unsigned long long& t0, int* err) {
+    if ((tries & 63) != 63) return false;
+    if (ld_volatile_int(err) != 0) return true;
+    const unsigned long long t = gtimer();
+    if (t0 == 0ull) t0 = t;
+    if (t - t0 <= kBarrierTimeoutNs) return false;
+    atomicCAS(err, 0, ACS_ERR_DEVICE_TIMEOUT);
+    return true;
+}
+
+// This lane's share of a reducing barrier: waits for the partials of CTAs b0,
+// b0 + step, ... and combines them in that order.  Returns false if a wait
+// expired.
+template <int NV>
+__device__ __forceinline__ bool gather_slots(const double* part, unsigned long long tag, int b0, int step, int size,
+                                             unsigned opmask, int* err, double (&x)[kMaxRed]) {
+    unsigned long long t0 = 0ull;
+    bool ok = true;
+    for (int b = b0; b < size && ok; b += step) {
+        const double* slot = part + (size_t)b * kPartStride;
+        double v[NV];
+        for (int tries = 0;; ++tries) {
+            bool all = true;
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                unsigned long long t;
+                v[k] = ld_slot(slot + 2 * k, t);
+                all = all && t == tag;
+            }
+            if (all) break;
+            if (wait_expired(tries, t0, err)) { ok = false; break; }
+        }
+#pragma unroll
+        for (int k = 0; k < NV; ++k) x[k] = (opmask >> k) & 1u ? fmax(x[k], v[k]) : x[k] + v[k];
+    }
+    return ok;
+}
+
+// The barrier up to the reduced values.
+//
+// Without values, thread 0 adds 1 to the team's monotonic arrival counter
+// with release semantics and spins (acquire) until the counter reaches
+// (generation) * (CTAs in the team): about two L2 round trips.
+//
+// With values the arrival is the value itself: warp 0 combines the warps of
+// this CTA, and its lane k writes (partial k, generation) to this CTA's slot;
+// lane l of warp w then waits for the slot of CTA 32 w + l, whose tag is the
+// news that that CTA has arrived, so that one L2 round trip after the last
+// arrival every CTA has every partial (counter, then partials: two).  The
+// counter is kept in step for the barriers without values.
+// A team of one CTA needs neither.  The caller follows with a CTA barrier.
+static __device__ __noinline__ void grid_reduce(int* err) {
     SyncShared& S = sync_smem();
-    __syncthreads();                                   // the phase's writes and S.blk are complete
+    __syncthreads();                                   // the phase's writes and S.wsum are complete
     const unsigned target = S.gen + 1u;
     const int nv = S.nv;
+    const int size = S.team_size;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int rank = S.team_rank, size = S.team_size;
-    if (size == 1) {
-        // writes of the phase are visible to the CTA after __syncthreads; the
-        // error word is still checked so that a failed problem stops
+    if (nv == 0) {
         if (threadIdx.x == 0) {
-            for (int k = 0; k < nv; ++k) S.out[k] = S.blk[k];
-            if (ld_volatile_int(err) != 0) S.fail = 1;
+            bool fail = false;
+            if (size > 1) {
+                red_add_release(S.bar, 1ull);
+                const unsigned long long want = (unsigned long long)target * size;
+                unsigned long long t0 = 0ull;
+                for (int tries = 0; ld_acquire64(S.bar) < want; ++tries)
+                    if (wait_expired(tries, t0, err)) { fail = true; break; }
+            }
+            if (fail || ld_volatile_int(err) != 0) S.fail = 1;
+            S.gen = target;
         }
-        __syncthreads();
-        const bool ok1 = S.fail == 0;
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        return;
+    }
+    const unsigned opmask = S.opmask;
+    if (warp == 0) {
+        const int nw = (int)(blockDim.x >> 5);
+        double x[kMaxRed];
+#pragma unroll
+        for (int k = 0; k < kMaxRed; ++k) {
+            x[k] = 0.0;
+            if (k < nv) x[k] = lane < nw ? S.wsum[lane][k] : ((opmask >> k) & 1u ? -INFINITY : 0.0);
+        }
+        warp_combine(x, nv, opmask, S.out);
+        if (size == 1) {
+            // the error word is still checked so that a failed problem stops
+            if (lane == 0) {
+                if (ld_volatile_int(err) != 0) S.fail = 1;
+                S.gen = target;
+                S.nv = 0;
+            }
+            __syncwarp();
+            return;
+        }
+    }
+    if (size == 1) return;
+    double* part = S.tpart + (target & 1u) * (2 * kMaxRed);
+    if (warp == 0) {
+        fence_gpu();                                    // the phase's writes come before the arrival
+        if (lane < (nv <= 3 ? nv : kMaxRed)) st_slot(part + (size_t)S.team_rank * kPartStride + 2 * lane, S.out[lane], target);
+        if (lane == 0) atomicAdd(S.bar, 1ull);
+    }
+    const int nwarp = min((size + 31) >> 5, (int)(blockDim.x >> 5));   // warps that gather
+    if (warp < nwarp) {
+        double x[kMaxRed];
+#pragma unroll
+        for (int k = 0; k < kMaxRed; ++k) x[k] = (opmask >> k) & 1u ? -INFINITY : 0.0;
+        bool ok;
+        const int b0 = warp * 32 + lane, step = nwarp * 32;
+        if (nv == 1) ok = gather_slots<1>(part, target, b0, step, size, opmask, err, x);
+        else if (nv == 2) ok = gather_slots<2>(part, target, b0, step, size, opmask, err, x);
+        else if (nv == 3) ok = gather_slots<3>(part, target, b0, step, size, opmask, err, x);
+        else ok = gather_slots<8>(part, target, b0, step, size, opmask, err, x);
+        ok = __all_sync(0xffffffffu, ok);
+        fence_gpu();                                    // and reads of what the others wrote after it
+        warp_combine(x, nv, opmask, S.gsum[warp]);
+        if (!ok && lane == 0) S.fail = 1;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < nv) {
+            const bool mx = (opmask >> lane) & 1u;
+            double x = S.gsum[0][lane];
+            for (int w = 1; w < nwarp; ++w) x = mx ? fmax(x, S.gsum[w][lane]) : x + S.gsum[w][lane];
+            S.out[lane] = x;
+        }
+        if (lane == 0) {
+            if (ld_volatile_int(err) != 0) S.fail = 1;
             S.gen = target;
             S.nv = 0;
         }
-        return ok1;
+        __syncwarp();
     }
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < nv; ++k) S.tpart[rank * kMaxRed + k] = S.blk[k];
-        red_add_release(S.bar, 1ull);
-        const unsigned long long want = (unsigned long long)target * size;
-        const unsigned long long t0 = gtimer();
-        int spins = 0;
-        while (ld_acquire64(S.bar) < want) {
-            if (++spins == 64) {
-                spins = 0;
-                if (ld_volatile_int(err) != 0) { S.fail = 1; break; }
-                if (gtimer() - t0 > kBarrierTimeoutNs) {
-                    atomicCAS(err, 0, ACS_ERR_DEVICE_TIMEOUT);
-                    S.fail = 1;
-                    break;
-                }
-            }
-        }
-        if (ld_volatile_int(err) != 0) S.fail = 1;
-    }
+}
+
+// Barrier and reduction, then post(S.out) in warp 0 (every lane, the same
+// values; post writes what the loop reads to shared memory).
+template <typename Post>
+__device__ __forceinline__ bool grid_sync_post(int* err, const Post& post) {
+    grid_reduce(err);
+    SyncShared& S = sync_smem();
+    if (threadIdx.x < 32) post(S.out);
     __syncthreads();
-    if (nv > 0) {
-        // gather every CTA's partials, combine in CTA order: lanes by a fixed
-        // shuffle tree, then the warps in order
-        const int b = threadIdx.x;
-        if (b < size)
-            for (int k = 0; k < nv; ++k) S.gath[k][b] = __ldcg(S.tpart + b * kMaxRed + k);
-        __syncthreads();
-        const int nwarp = (size + 31) >> 5;
-        if (warp < nwarp) {
-            for (int k = 0; k < nv; ++k) {
-                const int opk = S.op[k];
-                double x = (b < size) ? S.gath[k][b] : (opk ? -INFINITY : 0.0);
-                x = opk ? warp_max(x) : warp_sum(x);
-                if (lane == 0) S.wsum[warp][k] = x;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < nv) {
-            const int k = threadIdx.x;
-            const int opk = S.op[k];
-            double x = S.wsum[0][k];
-            for (int w = 1; w < nwarp; ++w) x = opk ? fmax(x, S.wsum[w][k]) : x + S.wsum[w][k];
-            S.out[k] = x;
-        }
-    }
-    __syncthreads();
-    const bool ok = S.fail == 0;
-    __syncthreads();                                   // everyone has read S.fail and S.out is final
-    if (threadIdx.x == 0) {
-        S.gen = target;
-        S.nv = 0;
-    }
-    return ok;
+    return S.fail == 0;
+}
+__device__ __forceinline__ bool grid_sync(int* err) {
+    return grid_sync_post(err, [](const double*) {});
 }
 
 // Values reduced at the last grid_sync.
@@ -904,15 +1089,11 @@ __device__ __noinline__ void phase_cond_o(const IterParams<T>& P) {
     block_partials<3>(v, op, P.partials);
 }
 
-// Exponent range of step 11 over the finite positive o.  An o of 0, inf or
+// Exponent range (CondRange) of step 11 over the finite positive o.  An o of 0, inf or
 // nan (x_h = ||xbar||, z_h = 0, or both) carries no scale: it takes the
 // limit of the rule under the e^t cap -- the smallest scale for o = 0, the
 // largest for o = inf, the geometric middle for nan.  With no finite
 // positive o at all, O = I.
-struct CondRange {
-    double alpha, lmin, lmax;
-    bool any;
-};
 __device__ __forceinline__ double cond_scale(double lo, const CondRange& R) {
     if (!R.any) return 1.0;
     double e = lo;
@@ -1144,14 +1325,48 @@ __device__ __noinline__ void phase_cg_A_cb(const IterParams<T>& P) {
     cb_pass(P.Acb, P.V.t, &P.ctl->err);
 }
 
+// Scalars of a Chronopoulos-Gear step, in warp 0 at the barriers of the CG:
+// after M u (delta = u'Mu), beta and alpha of step k (broke: p'Mp <= 0 in finite
+// precision, the solve has reached its attainable accuracy or M is singular
+// along p) ...
+__device__ __forceinline__ void cg_step_scalars(double delta, int k) {
+    LoopScalars& L = sync_smem().lp;
+    const double beta = (k == 0) ? 0.0 : L.gam / L.gam_prev;
+    const double denom = delta - ((k == 0) ? 0.0 : beta * L.gam / L.alpha_prev);
+    const double alpha = L.gam / denom;
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        L.broke = !(denom > 0.0);
+        L.alpha = alpha;
+        L.beta = beta;
+    }
+}
+// ... and after the vector step (gn = r'u): whether to go on.
+__device__ __forceinline__ void cg_next_scalars(double gn) {
+    LoopScalars& L = sync_smem().lp;
+    const double r = sqrt(fmax(gn, 0.0));
+    const int go = r > L.thr, far = r > 100.0 * L.thr;
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        L.gam_prev = L.gam;
+        L.alpha_prev = L.alpha;
+        L.gam = gn;
+        L.go = go;
+        L.far = far;
+        L.bad = !isfinite(gn);
+    }
+}
+
 // Chronopoulos-Gear vector step: p = u + beta p, sv = au + beta sv,
 // w += alpha p (FP64), r -= alpha sv, u = J^{-1} r; partial gamma = r'u.
 // au(i) = (M u)_i: stored by the A pass, or the partial sums of the
 // column-blocked A pass added in block order.
 template <typename T, bool CB>
-__device__ __noinline__ void phase_cg_vec(const IterParams<T>& P, double alpha, T beta) {
+__device__ __noinline__ void phase_cg_vec(const IterParams<T>& P) {
     double gam = 0.0;
     const Inner<T>& V = P.V;
+    const double alpha = sync_smem().lp.alpha;
+    const T beta = (T)sync_smem().lp.beta;
     const T a = (T)alpha;
     auto step = [&](int i, T aui) {
         const T pi = fma(beta, V.p[i], V.u[i]);
@@ -1231,13 +1446,13 @@ __device__ __forceinline__ void update_epi(const IterParams<T>& P, int j, double
 }
 
 // Partials of the update: ||s_new - s||^2, ||s_new||^2 and, for a
-// time-sliced solve, whether the deadline has passed (one clock read per
-// CTA, max-reduced, so every CTA of the team takes the same decision).
+// time-sliced solve, the CTAs that have seen the deadline pass (one clock
+// read per CTA, summed, so every CTA of the team takes the same decision).
 __device__ __forceinline__ void update_partials(double ds2, double ss2, bool update, double* partials) {
     const unsigned long long dl = sync_smem().deadline;
     const double over = (update && dl != 0ull && threadIdx.x == 0 && gtimer() > dl) ? 1.0 : 0.0;
     const double v[3] = {ds2, ss2, over};
-    const int op[3] = {0, 0, 1};
+    const int op[3] = {0, 0, 0};
     block_partials<3>(v, op, partials);
 }
 
@@ -1333,7 +1548,7 @@ __device__ __noinline__ void phase_kkt(const IterParams<T>& P) {
     const double* x = P.x;
     const double* z = P.z;
     const double* w = P.X.w;
-    const double inv_mu = 1.0 / P.mu;
+    const double inv_mu = P.inv_mu;
     {
         auto gather = [x](int j) { return x[j]; };
         auto epi = [&](int i, double sum) {
@@ -1744,7 +1959,7 @@ __device__ __noinline__ void phase_polish_jacobi(const IterParams<T>& P) {
 // y solve's start p = -O z_y, q = 0, g = O p, w = 0, b_tilde = 0.
 static __device__ __noinline__ void phase_polish_ystart(const IterParams<double>& P, const PolishOut& out) {
     const double* pw = out.pw;
-    const double inv_mu = 1.0 / P.mu;
+    const double inv_mu = P.inv_mu;
     auto gather = [pw, inv_mu](int i) { return pw[i] * inv_mu; };
     auto epi = [&](int j, double sum) {
         const double o = P.X.O[j];
@@ -1767,7 +1982,7 @@ static __device__ __noinline__ void phase_polish_ystart(const IterParams<double>
 // z~ = c - A'(pw / mu).
 static __device__ __noinline__ void phase_polish_z(const IterParams<double>& P, const PolishOut& out) {
     const double* pw = out.pw;
-    const double inv_mu = 1.0 / P.mu;
+    const double inv_mu = P.inv_mu;
     auto gather = [pw, inv_mu](int i) { return pw[i] * inv_mu; };
     auto epi = [&](int j, double sum) { out.pz[j] = P.c[j] - sum; };
     sell_rows<double>(P.AT, gather, epi);
@@ -1850,27 +2065,40 @@ __device__ __noinline__ void phase_polish_rhs(const IterParams<T>& P) {
 template <typename T>
 __device__ bool polish_solve(const IterParams<double>& P, const IterParams<T>& PT, int rounds, double rel,
                              bool dense, long long& cg_total) {
-    double gam_last = INFINITY, target = 0.0;
+    LoopScalars& L = sync_smem().lp;
+    double gam_last = INFINITY;
     for (int round = 0; round < rounds; ++round) {
         if (round > 0) {
             phase_polish_q(P);
             if (!grid_sync(&P.ctl->err)) return false;
         }
         phase_polish_rhs(PT);
-        if (!grid_sync(&P.ctl->err)) return false;
-        double gam, floor_r;
-        {
-            double t2[2];
-            const int op[2] = {0, 0};
-            grid_combine<2>(P.partials, op, t2);
-            gam = t2[0];
-            floor_r = 64.0 * 0x1p-52 * sqrt(fmax(t2[1], 0.0));
-        }
-        if (!isfinite(gam) || !isfinite(floor_r)) return false;
-        if (round == 0) target = rel * sqrt(fmax(gam, 0.0));
-        floor_r = fmax(floor_r, target);
-        if (!(sqrt(fmax(gam, 0.0)) > floor_r) || (round > 0 && gam > 0.01 * gam_last)) break;
-        gam_last = gam;
+        // an FP32 correction goes down to ~1e-5 of its round's residual; the
+        // next round's FP64 residual refines it
+        if (!grid_sync_post(&P.ctl->err, [&](const double* t2) {
+                const double gam = t2[0], gn = sqrt(fmax(gam, 0.0));
+                double floor_r = 64.0 * 0x1p-52 * sqrt(fmax(t2[1], 0.0));
+                const double target = round == 0 ? rel * gn : L.target;
+                const int bad = !isfinite(gam) || !isfinite(floor_r);
+                floor_r = fmax(floor_r, target);
+                const double thr = fmax((sizeof(T) == 4 ? 1e-5 : 1e-13) * sqrt(gam), floor_r);
+                const int broke = !(gn > floor_r) || (round > 0 && gam > 0.01 * gam_last);
+                __syncwarp();
+                if ((threadIdx.x & 31) == 0) {
+                    L.gam = gam;
+                    L.target = target;
+                    L.thr = thr;
+                    L.gam_prev = L.alpha_prev = 1.0;
+                    L.best = L.best_ref = gam;
+                    L.bad = bad;
+                    L.broke = broke;
+                    L.go = gn > thr;
+                }
+            }))
+            return false;
+        if (L.bad) return false;
+        if (L.broke) break;
+        gam_last = L.gam;
         if (sizeof(T) == 8 && dense) {                 // one exact correction: dw = X'(X r0)
             phase_dense_y(P);
             if (!grid_sync(&P.ctl->err)) return false;
@@ -1879,41 +2107,32 @@ __device__ bool polish_solve(const IterParams<double>& P, const IterParams<T>& P
             ++cg_total;
             continue;
         }
-        // an FP32 correction goes down to ~1e-5 of its round's residual; the
-        // next round's FP64 residual refines it
-        const double thr = fmax((sizeof(T) == 4 ? 1e-5 : 1e-13) * sqrt(gam), floor_r);
-        double gam_prev = 1.0, alpha_prev = 1.0;
-        // and, should the floor underestimate that part, the round ends
-        // when the smallest residual so far has not halved in kPolishWindow
-        // iterations
-        double best = gam, best_ref = gam;
+        // should the floor underestimate that part, the round ends when the
+        // smallest residual so far has not halved in kPolishWindow iterations
         int k = 0;
-        while (sqrt(fmax(gam, 0.0)) > thr && k < P.cg_max) {
-            double dl[1];
-            const int op1[1] = {0};
+        while (L.go && k < P.cg_max) {
             phase_polish_cg_At(PT);
             if (!grid_sync(&P.ctl->err)) return false;
             phase_cg_A(PT);
-            if (!grid_sync(&P.ctl->err)) return false;
-            grid_combine<1>(P.partials, op1, dl);
-            const double beta = (k == 0) ? 0.0 : gam / gam_prev;
-            const double denom = dl[0] - ((k == 0) ? 0.0 : beta * gam / alpha_prev);
-            if (!(denom > 0.0)) break;                  // attainable accuracy reached
-            const double alpha = gam / denom;
-            phase_cg_vec<T, false>(PT, alpha, (T)beta);
-            if (!grid_sync(&P.ctl->err)) return false;
-            double gn[1];
-            grid_combine<1>(P.partials, op1, gn);
-            gam_prev = gam;
-            alpha_prev = alpha;
-            gam = gn[0];
+            if (!grid_sync_post(&P.ctl->err, [&](const double* dl) { cg_step_scalars(dl[0], k); })) return false;
+            if (L.broke) break;                         // attainable accuracy reached
+            phase_cg_vec<T, false>(PT);
+            if (!grid_sync_post(&P.ctl->err, [&](const double* gn) {
+                    cg_next_scalars(gn[0]);
+                    const double best = fmin(L.best, gn[0]);
+                    const bool window = (k + 1) % kPolishWindow == 0;
+                    const int stuck = window && best > 0.5 * L.best_ref;
+                    __syncwarp();
+                    if ((threadIdx.x & 31) == 0) {
+                        L.best = best;
+                        if (window) L.best_ref = best;
+                        L.broke = stuck;
+                    }
+                }))
+                return false;
             ++k;
-            if (!isfinite(gam)) return false;
-            best = fmin(best, gam);
-            if (k % kPolishWindow == 0) {
-                if (best > 0.5 * best_ref) break;
-                best_ref = best;
-            }
+            if (L.bad) return false;
+            if (L.broke) break;
         }
         cg_total += k;
     }
@@ -2034,12 +2253,16 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
     const bool cbcg = sizeof(T) == 4 && P.Acb.nblocks > 0 && P.ATcb.nblocks > 0;
     int outer32_end = __ldcg(&ctl->outer32_end);
     bool outer32 = cbcg && P.outer32 != 0 && outer32_end == 0;
-    double best_mx = INFINITY;
-    int flat_checks = 0;
-    double res[6];
-    for (int i = 0; i < 6; ++i) res[i] = __ldcg(&ctl->res[i]);
-    double ds = __ldcg(&ctl->ds), snorm = __ldcg(&ctl->snorm);
-    double eta = __ldcg(&ctl->eta);
+    LoopScalars& L = sync_smem().lp;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 6; ++i) L.res[i] = __ldcg(&ctl->res[i]);
+        L.ds = __ldcg(&ctl->ds);
+        L.snorm = __ldcg(&ctl->snorm);
+        L.eta = __ldcg(&ctl->eta);
+        L.best_mx = INFINITY;
+        L.flat_checks = 0;
+    }
+    __syncthreads();
     bool ok = true;
     // cached projection operator (FP64 loops only); a factorisation that fails
     // (M singular: rank-deficient A) hands this solve to the CG projection
@@ -2072,10 +2295,12 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
     // ends at a polish level)
     const bool outer32_l2 = sizeof(T) == 4 && P.outer32_l2 != 0 && !cbcg && P.A.v32 && P.AT.v32;
 
-// grid barrier that ends phase `ph`; leaves the enclosing loop on error
-#define ACS_SYNC(ph)                                                      \
+// grid barrier that ends phase `ph`, with the scalars of the next phases in
+// its post function; leaves the enclosing loop on error
+#define ACS_SYNC(ph) ACS_SYNC_POST(ph, [](const double*) {})
+#define ACS_SYNC_POST(ph, ...)                                            \
     {                                                                     \
-        if (!(ok = grid_sync(&ctl->err))) break;                                \
+        if (!(ok = grid_sync_post(&ctl->err, __VA_ARGS__))) break;        \
         if (clock_owner) {                                                \
             const unsigned long long t_ = gtimer();                       \
             s_ph_ns[ph] += t_ - s_last;                                   \
@@ -2103,19 +2328,18 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         }
         if (cond) {                                             // steps 5-14
             phase_cond_o(P);
-            ACS_SYNC(PH_COND_O);
-            double mm[3];
-            const int op[3] = {1, 1, 0};
-            grid_combine<3>(P.partials, op, mm);
-            CondRange R;
-            R.any = mm[2] > 0.0;                               // some o finite and positive
-            R.lmax = mm[0];
-            R.lmin = -mm[1];
-            const double spread = R.lmax - R.lmin;             // log max o - log min o
-            if (!R.any) R.alpha = 0.0;
-            else if (!(spread > 0.0)) R.alpha = 1.0;
-            else R.alpha = fmin(1.0, P.t_cond / spread);
-            phase_cond_apply(P, R, true, true);
+            ACS_SYNC_POST(PH_COND_O, [&](const double* mm) {
+                CondRange R;
+                R.any = mm[2] > 0.0;                           // some o finite and positive
+                R.lmax = mm[0];
+                R.lmin = -mm[1];
+                const double spread = R.lmax - R.lmin;         // log max o - log min o
+                if (!R.any) R.alpha = 0.0;
+                else if (!(spread > 0.0)) R.alpha = 1.0;
+                else R.alpha = fmin(1.0, P.t_cond / spread);
+                if (threadIdx.x == 0) L.range = R;
+            });
+            phase_cond_apply(P, L.range, true, true);
             ACS_SYNC(PH_COND_APPLY);
             ++ncond;
         } else if (refresh) {
@@ -2125,11 +2349,10 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         if (cond || refresh) {
             phase_btilde(P);
             ++nA64;
-            ACS_SYNC(PH_BTILDE);
-            double bb[1];
-            const int op[1] = {0};
-            grid_combine<1>(P.partials, op, bb);
-            if (bb[0] > 0.0) { atomicCAS(&ctl->err, 0, ACS_ERR_FACTOR); ok = false; break; }
+            ACS_SYNC_POST(PH_BTILDE, [&](const double* bb) {
+                if (threadIdx.x == 0) L.bad = bb[0] > 0.0;
+            });
+            if (L.bad) { atomicCAS(&ctl->err, 0, ACS_ERR_FACTOR); ok = false; break; }
             if (cond) factor_ok = false;                    // O changed: the factor is stale
             if (dense && factor_kept && !cond) {
                 factor_kept = false;                        // resumed: the cached factor is current
@@ -2191,39 +2414,42 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                 ++nAT64;
                 ACS_SYNC(PH_QREFRESH);
             }
+            // the step-relative rule needs a previous step in the same scaling;
+            // on the first iteration and whenever O changes only the floors apply
+            auto start_cg = [&](const double* t1) {
+                const double gam = t1[0], g = sqrt(fmax(gam, 0.0));
+                const double rel = (isfinite(L.ds) && !cond && round == 0) ? L.eta * L.ds : 0.0;
+                const double thr = fmax(fmax(rel, P.cg_tol * L.snorm), P.cg_relfloor * g);
+                const int go = g > thr, far = g > 100.0 * thr;
+                if (threadIdx.x == 0) {
+                    L.gam = gam;
+                    L.thr = thr;
+                    L.gam_prev = L.alpha_prev = 1.0;
+                    L.bad = !isfinite(gam);
+                    L.go = go;
+                    L.far = far;
+                }
+            };
             if (outer32) {                                      // r0 from an FP32 product
                 phase_rhs_cb(P);
                 ++nA32;
                 ACS_SYNC(PH_RHS);
                 phase_rhs_comb(P);
-                ACS_SYNC(PH_RHS_COMB);
+                ACS_SYNC_POST(PH_RHS_COMB, start_cg);
             } else if (outer32_l2) {
                 phase_rhs_f32(P);                               // r0 from an FP32 product
                 ++nA32;
-                ACS_SYNC(PH_RHS);
+                ACS_SYNC_POST(PH_RHS, start_cg);
             } else {
                 phase_rhs(P);                                   // r0 in FP64
                 ++nA64;
-                ACS_SYNC(PH_RHS);
+                ACS_SYNC_POST(PH_RHS, start_cg);
             }
-            double gam;
-            {
-                double t1[1];
-                const int op[1] = {0};
-                grid_combine<1>(P.partials, op, t1);
-                gam = t1[0];
-            }
-            if (!isfinite(gam)) { status = ACS_ERR_NUMERICAL; break; }
-            // the step-relative rule needs a previous step in the same scaling;
-            // on the first iteration and whenever O changes only the floors apply
-            const double rel = (isfinite(ds) && !cond && round == 0) ? eta * ds : 0.0;
-            const double thr = fmax(fmax(rel, P.cg_tol * snorm), P.cg_relfloor * sqrt(fmax(gam, 0.0)));
-            double gam_prev = 1.0, alpha_prev = 1.0;
+            if (L.bad) { status = ACS_ERR_NUMERICAL; break; }
             int k = 0;
             bool broke = false;
-            while (sqrt(fmax(gam, 0.0)) > thr && k < P.cg_max) {
-                double dl[1];
-                const int op1[1] = {0};
+            while (L.go && k < P.cg_max) {
+                auto step_scalars = [&](const double* dl) { cg_step_scalars(dl[0], k); };
                 if (cbcg) {
                     // column-blocked passes: u'Mu = ||A_hat'u||^2 is known after
                     // the first half, the second half's sums are combined in the
@@ -2232,49 +2458,37 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                     ++nAT;
                     ACS_SYNC(PH_CG_AT);
                     phase_cg_tcomb(P);                          // t = O^2 A'u, u'Mu
-                    ACS_SYNC(PH_CG_TCOMB);
-                    grid_combine<1>(P.partials, op1, dl);
+                    ACS_SYNC_POST(PH_CG_TCOMB, step_scalars);
                 } else {
                     phase_cg_At(P);                             // t = O^2 A' u
                     ++nAT;
                     ACS_SYNC(PH_CG_AT);
                     phase_cg_A(P);                              // au = A t = M u
                     ++nA;
-                    ACS_SYNC(PH_CG_A);
-                    grid_combine<1>(P.partials, op1, dl);
+                    ACS_SYNC_POST(PH_CG_A, step_scalars);
                 }
-                const double beta = (k == 0) ? 0.0 : gam / gam_prev;
-                const double denom = dl[0] - ((k == 0) ? 0.0 : beta * gam / alpha_prev);
-                if (!(denom > 0.0)) {
-                    // p'Mp <= 0 in finite precision: the solve has reached its
-                    // attainable accuracy (or M is singular along p); keep w --
-                    // the next FP64 residual carries on from it
+                if (L.broke) {
+                    // keep w -- the next FP64 residual carries on from it
                     broke = true;
                     break;
                 }
-                const double alpha = gam / denom;
                 if (cbcg) {
                     phase_cg_A_cb(P);                           // partial sums of A t = M u
                     ++nA;
                     ACS_SYNC(PH_CG_A);
-                    phase_cg_vec<T, true>(P, alpha, (T)beta);
+                    phase_cg_vec<T, true>(P);
                 } else {
-                    phase_cg_vec<T, false>(P, alpha, (T)beta);
+                    phase_cg_vec<T, false>(P);
                 }
-                ACS_SYNC(PH_CG_VEC);
-                double gn[1];
-                grid_combine<1>(P.partials, op1, gn);
-                gam_prev = gam;
-                alpha_prev = alpha;
-                gam = gn[0];
+                ACS_SYNC_POST(PH_CG_VEC, [&](const double* gn) { cg_next_scalars(gn[0]); });
                 ++k;
-                if (!isfinite(gam)) { status = ACS_ERR_NUMERICAL; break; }
+                if (L.bad) { status = ACS_ERR_NUMERICAL; break; }
             }
             if (!ok || status == ACS_ERR_NUMERICAL) break;
             cg_total += k;
             win_cg += k;
             // an FP32 solve that stalls far above its target cannot refine this M
-            if ((broke || k >= P.cg_max) && sqrt(fmax(gam, 0.0)) > 100.0 * thr) trouble = true;
+            if ((broke || k >= P.cg_max) && L.far) trouble = true;
         }
         if (!ok || status == ACS_ERR_NUMERICAL) break;
 
@@ -2283,53 +2497,67 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         // step 17 of the next iteration in this pass's epilogue (orthant-only,
         // no extrapolation, no rescaling at the next iteration)
         const bool fuse_abs = P.n_soc == 0 && !P.admm && P.extrap == 0.0 && !in_schedule(P, lnext + 1);
+        // With exact projections the step norm ||s_l - s_{l-1}|| never grows
+        // between rescalings (the iteration map is firmly nonexpansive,
+        // Lemma 3); growth beyond what the allowed error explains means the
+        // CG error estimate (J-norm of the residual) is too optimistic for
+        // this M, so the rule is tightened for the rest of the solve.
+        // In the FP32 solve a factor below 1e-4 * cg_eta means the FP32
+        // correction cannot reach the accuracy this M needs: the solve
+        // continues with an FP64 correction solve instead.
+        auto end_step = [&](double d0, double d1) {
+            const double ds_new = sqrt(d0), sn = sqrt(d1);
+            const int bad = !isfinite(ds_new) || !isfinite(sn);
+            const double ds = L.ds;
+            double eta = L.eta;
+            int tr = 0;
+            if (!cond && isfinite(ds) && ds_new > (1.0 + 4.0 * eta) * ds && eta > 1e-8) {
+                if (sizeof(T) == 4 && eta <= 1e-4 * P.cg_eta * 1.0000001) tr = 1;
+                else eta *= 0.1;
+            }
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                L.snorm = sn;
+                L.bad = bad;
+                L.trouble = bad ? 0 : tr;
+                if (!bad) {
+                    L.eta = eta;
+                    L.ds = ds_new;
+                }
+            }
+        };
+        const bool two_parts = P.admm && P.n_soc > 0;            // the cones' share of the update follows
+        auto after_update = [&](const double* d2) {
+            if (threadIdx.x == 0) {
+                L.over = d2[2] > 0.0;
+                L.d0 = d2[0];
+                L.d1 = d2[1];
+            }
+            if (!two_parts) end_step(d2[0], d2[1]);
+        };
         if (outer32) {                                          // steps 18-21, FP32 product
             phase_update_cb(P);
             ++nAT32;
             ACS_SYNC(PH_UPDATE);
             phase_update_comb(P, want_xz, fuse_abs);
-            ACS_SYNC(PH_UPD_COMB);
+            ACS_SYNC_POST(PH_UPD_COMB, after_update);
         } else if (outer32_l2) {
             phase_update_f32(P, want_xz, fuse_abs);             // steps 18-21, FP32 product
             ++nAT32;
-            ACS_SYNC(PH_UPDATE);
+            ACS_SYNC_POST(PH_UPDATE, after_update);
         } else {
             phase_update(P, true, want_xz, fuse_abs);          // steps 18-21
             ++nAT64;
-            ACS_SYNC(PH_UPDATE);
+            ACS_SYNC_POST(PH_UPDATE, after_update);
         }
         abs_fused = fuse_abs;
-        {
-            double d2[3];
-            const int op[3] = {0, 0, 1};
-            grid_combine<3>(P.partials, op, d2);
-            if (P.admm && P.n_soc > 0) {                        // the cones' share of the update
-                phase_admm_soc(P, want_xz);
-                ACS_SYNC(PH_UPDATE);
-                double e2[2];
-                const int op2[2] = {0, 0};
-                grid_combine<2>(P.partials, op2, e2);
-                d2[0] += e2[0];
-                d2[1] += e2[1];
-            }
-            const double ds_new = sqrt(d2[0]);
-            snorm = sqrt(d2[1]);
-            over = d2[2] > 0.0;
-            if (!isfinite(ds_new) || !isfinite(snorm)) { status = ACS_ERR_NUMERICAL; l = lnext; break; }
-            // With exact projections the step norm ||s_l - s_{l-1}|| never grows
-            // between rescalings (the iteration map is firmly nonexpansive,
-            // Lemma 3); growth beyond what the allowed error explains means the
-            // CG error estimate (J-norm of the residual) is too optimistic for
-            // this M, so the rule is tightened for the rest of the solve.
-            // In the FP32 solve a factor below 1e-4 * cg_eta means the FP32
-            // correction cannot reach the accuracy this M needs: the solve
-            // continues with an FP64 correction solve instead.
-            if (!cond && isfinite(ds) && ds_new > (1.0 + 4.0 * eta) * ds && eta > 1e-8) {
-                if (sizeof(T) == 4 && eta <= 1e-4 * P.cg_eta * 1.0000001) trouble = true;
-                else eta *= 0.1;
-            }
-            ds = ds_new;
+        over = L.over != 0;
+        if (two_parts) {
+            phase_admm_soc(P, want_xz);
+            ACS_SYNC_POST(PH_UPDATE, [&](const double* e2) { end_step(L.d0 + e2[0], L.d1 + e2[1]); });
         }
+        if (L.bad) { status = ACS_ERR_NUMERICAL; l = lnext; break; }
+        if (L.trouble) trouble = true;
         l = lnext;
         ++win_it;
         if (sizeof(T) == 4 && trouble && P.switch_ok) { status = ST_SWITCH; break; }
@@ -2339,38 +2567,44 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
             ++nA64;
             ++nAT64;
             ++nchk;
-            ACS_SYNC(PH_KKT);
-            double r8[8];
-            const int op[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            grid_combine<8>(P.partials, op, r8);
-            res[0] = sqrt(r8[0]) / (1.0 + P.bnorm);
-            res[1] = sqrt(r8[1]) / (1.0 + P.cnorm);
-            res[2] = fabs(r8[2] - r8[3]) / (1.0 + fabs(r8[2]) + fabs(r8[3]));
-            res[3] = fmax(sqrt(r8[4]), sqrt(r8[5])) / (1.0 + fmax(sqrt(r8[6]), sqrt(r8[7])));
-            res[4] = r8[2];
-            res[5] = r8[3];
-            const double mx = fmax(fmax(res[0], res[1]), fmax(res[2], res[3]));
-            if (!isfinite(mx)) { status = ACS_ERR_NUMERICAL; break; }
-            if (mx <= P.tol) { status = ACS_SOLVED; break; }
             // FP32 outer passes end once the residuals reach outer32_tol, or
             // once they stop falling (the FP32 products' rounding floor): the
             // rest of the solve runs the FP64 passes from the same iterate
-            if (outer32) {
-                if (mx < 0.9 * best_mx) {
-                    best_mx = mx;
-                    flat_checks = 0;
-                } else {
-                    ++flat_checks;
+            ACS_SYNC_POST(PH_KKT, [&](const double* r8) {
+                const double rp = sqrt(r8[0]) / (1.0 + P.bnorm);
+                const double rd = sqrt(r8[1]) / (1.0 + P.cnorm);
+                const double rg = fabs(r8[2] - r8[3]) / (1.0 + fabs(r8[2]) + fabs(r8[3]));
+                const double rc = fmax(sqrt(r8[4]), sqrt(r8[5])) / (1.0 + fmax(sqrt(r8[6]), sqrt(r8[7])));
+                const double mx = fmax(fmax(rp, rd), fmax(rg, rc));
+                if (threadIdx.x == 0) {
+                    L.res[0] = rp;
+                    L.res[1] = rd;
+                    L.res[2] = rg;
+                    L.res[3] = rc;
+                    L.res[4] = r8[2];
+                    L.res[5] = r8[3];
+                    L.bad = !isfinite(mx);
+                    L.solved = mx <= P.tol;
+                    if (mx < 0.9 * L.best_mx) {
+                        L.best_mx = mx;
+                        L.flat_checks = 0;
+                    } else {
+                        ++L.flat_checks;
+                    }
+                    L.end32 = mx <= P.outer32_tol || L.flat_checks >= kOuter32FlatChecks;
                 }
-                if (mx <= P.outer32_tol || flat_checks >= kOuter32FlatChecks) {
-                    outer32 = false;
-                    outer32_end = l;
-                }
+            });
+            if (L.bad) { status = ACS_ERR_NUMERICAL; break; }
+            if (L.solved) { status = ACS_SOLVED; break; }
+            if (outer32 && L.end32) {
+                outer32 = false;
+                outer32_end = l;
             }
         }
         if (over && l < P.max_iter) { status = ST_PAUSED; break; }
     }
 #undef ACS_SYNC
+#undef ACS_SYNC_POST
 
     if (clock_owner) {
         const int err = ld_volatile_int(&ctl->err);
@@ -2378,10 +2612,10 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         if (status == ST_SWITCH && err == 0) ctl->switched_at = l;
         ctl->l = l;
         ctl->cg_iters += cg_total;
-        for (int i = 0; i < 6; ++i) ctl->res[i] = res[i];
-        ctl->ds = ds;
-        ctl->snorm = snorm;
-        ctl->eta = eta;
+        for (int i = 0; i < 6; ++i) ctl->res[i] = L.res[i];
+        ctl->ds = L.ds;
+        ctl->snorm = L.snorm;
+        ctl->eta = L.eta;
         ctl->n_cg_A += nA;
         ctl->n_cg_AT += nAT;
         ctl->n_64_A += nA64;

@@ -16,6 +16,11 @@ namespace acs {
 constexpr int kThreads = 1024;          // threads per CTA of the persistent kernel
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRed = 8;              // doubles reduced per grid reduction
+// A CTA's partials, (value, generation) pairs: two sets, used by barriers of
+// even and odd generation, so
+// that a CTA that has passed a barrier and reaches the next one does not
+// overwrite what a slower CTA still reads.
+constexpr int kPartStride = 4 * kMaxRed;
 constexpr unsigned long long kBarrierTimeoutNs = 2000000000ull;   // 2 s per barrier
 // FP32 outer passes end after this many KKT checks without a 10 % fall of the
 // largest residual (they have reached the rounding floor of FP32 products)
@@ -135,13 +140,13 @@ struct IterParams {
     Inner<T> V;
     double* x; double* z;                             // FP64 iterates (steps 20-21)
     double* ocone;                                    // log o per cone (orthant coords first)
-    double* partials;                                 // [gridDim.x * kMaxRed]
+    double* partials;                                 // [gridDim.x * kPartStride]
     unsigned* flags;                                  // [gridDim.x] barrier arrival flags
     unsigned* release;                                // barrier release flag
     double* bcast;                                    // [kMaxRed] reduced values
     Control* ctl;
     // settings
-    double mu, t_cond;
+    double mu, inv_mu, t_cond;
     int cond_first, cond_period;
     const int* cond_list; int n_cond_list;
     int check_every, max_iter;

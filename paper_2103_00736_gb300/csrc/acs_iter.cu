@@ -89,6 +89,8 @@ pass_bench_kernel(const __grid_constant__ IterParams<float> P, const __grid_cons
     if (P.Acb.nblocks > 0) cb_init();
     const bool cbA = P.Acb.nblocks > 0, cbT = P.ATcb.nblocks > 0;
     const bool l2A = P.A.v32 != nullptr, l2T = P.AT.v32 != nullptr;
+    if (threadIdx.x == 0) sync_smem().lp.alpha = sync_smem().lp.beta = 0.0;   // the vector step leaves w, r
+    __syncthreads();
     const unsigned long long t0 = gtimer();
     int r = 0;
     for (; r < reps; ++r) {
@@ -96,10 +98,10 @@ pass_bench_kernel(const __grid_constant__ IterParams<float> P, const __grid_cons
             case 0: if (cbT) phase_cg_At_cb(P); break;
             case 1: if (cbT) phase_cg_tcomb(P); break;
             case 2: if (cbA) phase_cg_A_cb(P); break;
-            case 3: if (cbA) phase_cg_vec<float, true>(P, 0.0, 0.f); break;
+            case 3: if (cbA) phase_cg_vec<float, true>(P); break;
             case 4: if (l2T) phase_cg_At(P); break;
             case 5: if (l2A) phase_cg_A(P); break;
-            case 6: if (l2A) phase_cg_vec<float, false>(P, 0.0, 0.f); break;
+            case 6: if (l2A) phase_cg_vec<float, false>(P); break;
             case 7: phase_rhs(P64); break;
             case 8: phase_update(P64, false, false); break;
             case 10: phase_abs(P64, 0.0); break;
@@ -157,7 +159,9 @@ __global__ void __launch_bounds__(kThreads, 1) polish_kernel(const __grid_consta
 // ---------------------------------------------------------------------------
 
 // the grid barrier's counters, restarted for a launch outside a solve
-__global__ void reset_barrier(Control* ctl) {
+__global__ void reset_barrier(Control* ctl, double* partials, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) partials[i] = 0.0;   // tags of generation 0
+    if (threadIdx.x != 0) return;
     ctl->bar_count = 0;
     ctl->bar_gen = 0;
     ctl->bar_count64 = 0;
@@ -176,8 +180,10 @@ __global__ void init_identity_heads(double* x, double* z, int n_orth, const int*
     if (j < n_orth) { x[j] = 1.0; z[j] = 1.0; }
     if (j < n_soc) { const int a = soc_off[j]; x[a] = 1.0; z[a] = 1.0; }
 }
-__global__ void reset_flags(unsigned* flags, unsigned* release, int n) {
+// (the partials' generation tags too: a solve's barriers count from 1)
+__global__ void reset_flags(unsigned* flags, unsigned* release, int n, double* partials, int np) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) flags[i] = 0u;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) partials[i] = 0.0;
     if (blockIdx.x == 0 && threadIdx.x == 0) *release = 0u;
 }
 __global__ void reset_control(Control* ctl, int l, double ds, double snorm, double eta) {
@@ -224,7 +230,7 @@ static IterParams<T> make_params(Problem* P, double tol, int max_iter, const Inn
     Q.partials = P->partials;
     Q.flags = P->flags; Q.release = P->release; Q.bcast = P->bcast;
     Q.ctl = P->ctl;
-    Q.mu = P->set.mu; Q.t_cond = P->set.t;
+    Q.mu = P->set.mu; Q.inv_mu = 1.0 / P->set.mu; Q.t_cond = P->set.t;
     Q.cond_first = P->set.cond_first; Q.cond_period = P->set.cond_period;
     Q.cond_list = P->cond_list; Q.n_cond_list = (int)P->cond_list_host.size();
     Q.check_every = P->set.check_every > 0 ? P->set.check_every : 1;
@@ -300,7 +306,8 @@ int pass_bench(Problem* P, int kind, int reps, int smem_bytes, double* us) {
             cudaSuccess ||
         per_sm < 1)
         return ACS_ERR_CUDA;
-    reset_flags<<<1, 256, 0, st>>>(P->flags, P->release, P->max_ctas);
+    reset_flags<<<8, 256, 0, st>>>(P->flags, P->release, P->max_ctas, P->partials,
+                                   std::max(P->grid32, P->grid64) * kPartStride);
     reset_control<<<1, 1, 0, st>>>(P->ctl, 0, INFINITY, 0.0, P->set.cg_eta);
     IterParams<float> Q = make_params<float>(P, 0.0, 1, P->V32);
     IterParams<double> Q64 = make_params<double>(P, 0.0, 1, P->V64);
@@ -323,7 +330,8 @@ int pass_bench(Problem* P, int kind, int reps, int smem_bytes, double* us) {
 
 int barrier_probe(Problem* P, int n, double* ns_per_barrier, int absent) {
     cudaStream_t st = P->stream;
-    reset_flags<<<1, 256, 0, st>>>(P->flags, P->release, P->max_ctas);
+    reset_flags<<<8, 256, 0, st>>>(P->flags, P->release, P->max_ctas, P->partials,
+                                   std::max(P->grid32, P->grid64) * kPartStride);
     reset_control<<<1, 1, 0, st>>>(P->ctl, 0, INFINITY, 0.0, P->set.cg_eta);
     double* d_out = P->bcast;
     void* args[] = {(void*)&P->ctl, (void*)&P->flags, (void*)&P->partials, (void*)&n, (void*)&d_out,
@@ -370,7 +378,7 @@ int launch_polish(Problem* P, int rounds, double rel) {
     if (cudaMemcpyAsync(P->pw, P->X.w, sizeof(double) * m, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemsetAsync(P->pres, 0, sizeof(double) * 16, st) != cudaSuccess)
         return ACS_ERR_CUDA;
-    reset_barrier<<<1, 1, 0, st>>>(P->ctl);
+    reset_barrier<<<1, 1024, 0, st>>>(P->ctl, P->partials, P->grid64 * kPartStride);
     if (cudaGetLastError() != cudaSuccess) return ACS_ERR_CUDA;
     IterParams<double> Q = make_params<double>(P, 0.0, 1, P->V64);
     Q.dense = 0;
@@ -414,7 +422,8 @@ int launch_solve(Problem* P, double tol, int max_iter) {
     const int n = P->n, m = P->m;
     const int big = n > m ? n : m;
     const int nb = (big + 255) / 256 > 4096 ? 4096 : (big + 255) / 256;
-    reset_flags<<<1, 256, 0, st>>>(P->flags, P->release, P->max_ctas);
+    reset_flags<<<8, 256, 0, st>>>(P->flags, P->release, P->max_ctas, P->partials,
+                                   std::max(P->grid32, P->grid64) * kPartStride);
     if (P->warm) reset_control<<<1, 1, 0, st>>>(P->ctl, P->warm_l, P->warm_ds, P->warm_snorm, P->warm_eta);
     else reset_control<<<1, 1, 0, st>>>(P->ctl, 0, INFINITY, 0.0, P->set.cg_eta);
     if (!P->warm) {

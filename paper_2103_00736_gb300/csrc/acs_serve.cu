@@ -432,6 +432,7 @@ double run_round(Server* S, int cls) {
     cudaMemsetAsync(S->d_t0, 0, sizeof(unsigned long long), st);
     cudaMemsetAsync(S->d_team_bar, 0, sizeof(unsigned long long) * S->max_ctas, st);
     cudaMemsetAsync(S->d_team_err, 0, sizeof(int) * S->max_ctas, st);
+    cudaMemsetAsync(S->d_team_part, 0, sizeof(double) * kPartStride * S->max_ctas, st);
     BatchArgs a{};
     a.count = (int)order.size();
     a.order = S->d_order;
@@ -625,7 +626,7 @@ int acs_server_create(const acs_settings* settings, const acs_server_config* cfg
     rc |= salloc(S, &S->d_head, 1);
     rc |= salloc(S, &S->d_mailbox, S->max_ctas);
     rc |= salloc(S, &S->d_team_bar, S->max_ctas);
-    rc |= salloc(S, &S->d_team_part, (size_t)S->max_ctas * kMaxRed);
+    rc |= salloc(S, &S->d_team_part, (size_t)S->max_ctas * kPartStride);
     rc |= salloc(S, &S->d_team_err, S->max_ctas);
     rc |= salloc(S, &S->d_cta, 3 * (size_t)S->max_ctas);
     rc |= salloc(S, &S->d_t0, 1);

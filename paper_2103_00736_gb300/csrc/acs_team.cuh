@@ -32,7 +32,7 @@ struct BatchArgs {
     int* head;                        // next position in order
     int* mailbox;                     // [teams] member posted by the team's rank 0
     unsigned long long* team_bar;     // [teams] barrier arrival counters
-    double* team_part;                // [CTAs * kMaxRed] partials
+    double* team_part;                // [CTAs * kPartStride] partials
     int* team_err;                    // [teams] barrier failures outside a member's solve
     double* dense;                    // [teams * 2 * dense_m2] scratch of the cached operator
     long long dense_m2;               // (largest m among members that use it)^2
@@ -75,6 +75,9 @@ __global__ void batch_reset(BatchArgs B, double eta0) {
 }
 
 __global__ void batch_reset_teams(BatchArgs B, int teams) {
+    // tags of generation 0: the teams' barriers count from 1
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < teams * B.g * kPartStride; i += gridDim.x * blockDim.x)
+        B.team_part[i] = 0.0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < teams; t += gridDim.x * blockDim.x) {
         B.team_bar[t] = 0ull;
         B.team_err[t] = 0;
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) batch_kernel(BatchArgs B)
         if (k < 0) return;
         const int rank = __ldg(B.cta_rank + blockIdx.x), g = __ldg(B.cta_g + blockIdx.x);
         const int base = (int)blockIdx.x - rank;
-        team_set(rank, g, B.team_bar + base, B.team_part + (size_t)base * kMaxRed, nullptr, nullptr);
+        team_set(rank, g, B.team_bar + base, B.team_part + (size_t)base * kPartStride, nullptr, nullptr);
         sync_init(0u);
         const unsigned long long deadline = launch_deadline(B);
         run_member(B, __ldg(B.order + k), nullptr, deadline);
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) batch_kernel(BatchArgs B)
     }
     const int team = (int)blockIdx.x / B.g, rank = (int)blockIdx.x % B.g;
     double* scratch = B.dense ? B.dense + (size_t)team * 2 * B.dense_m2 : nullptr;
-    team_set(rank, B.g, B.team_bar + team, B.team_part + (size_t)team * B.g * kMaxRed, scratch,
+    team_set(rank, B.g, B.team_bar + team, B.team_part + (size_t)team * B.g * kPartStride, scratch,
              scratch ? scratch + B.dense_m2 : nullptr);
     sync_init(0u);
     __shared__ int s_k;
@@ -323,7 +326,7 @@ IterParams<T> member_params(const acs_settings& set, const int* d_cond_list, int
     Q.x = M.x; Q.z = M.z; Q.ocone = M.ocone;
     Q.partials = nullptr; Q.flags = nullptr; Q.release = nullptr; Q.bcast = nullptr;
     Q.ctl = nullptr;
-    Q.mu = set.mu; Q.t_cond = set.t;
+    Q.mu = set.mu; Q.inv_mu = 1.0 / set.mu; Q.t_cond = set.t;
     Q.cond_first = set.cond_first; Q.cond_period = set.cond_period;
     Q.cond_list = d_cond_list; Q.n_cond_list = n_cond_list;
     Q.check_every = set.check_every > 0 ? set.check_every : 1;
