@@ -1230,6 +1230,14 @@ __device__ __forceinline__ void rhs_epi(const IterParams<T>& P, int i, double su
     gam += (double)r * (double)u;
 }
 
+// The residual alone, for the cached operator (no CG, no reduction).
+template <typename T>
+__device__ __noinline__ void phase_rhs_plain(const IterParams<T>& P) {
+    const double* g = P.X.g;
+    sell_rows<double>(P.A, [g](int j) { return g[j]; },
+                      [&](int i, double sum) { P.V.r[i] = (T)(P.X.btil[i] - sum); });
+}
+
 template <typename T>
 __device__ __noinline__ void phase_rhs(const IterParams<T>& P) {
     double gam = 0.0;
@@ -1612,8 +1620,9 @@ __device__ __noinline__ void phase_kkt(const IterParams<T>& P) {
 // correction of every iteration, dw = M^{-1} r0 = X' (X r0), is exact up to
 // rounding, like the oracle's dense solve, and costs two triangular matrix-
 // vector products with no sequential dependence.
-// Storage: M row-major [m x m] (lower triangle used, overwritten by L);
-// X column-major (X[c * m + i] = (L^{-1})_{ic}, i >= c).
+// Storage, both m x m: dX holds X row-major (lower triangle), dM first M
+// row-major (lower triangle, overwritten by L) and, once X is complete, X' row-
+// major (upper triangle), so that both products read rows.
 
 // M = A O^2 A' (lower triangle), from row i of A and the columns of A it
 // touches (rows of A'): M_ik = sum_j O_j^2 a_ij a_kj.  Warp per row i, the
@@ -1733,168 +1742,439 @@ __device__ __noinline__ void phase_dense_assemble(const IterParams<T>& P) {
 // right-hand side (b in range(A)) this solves the remaining independent
 // equations, which imply the dropped one.  A pivot negative beyond rounding
 // or not a number fails the factorisation.
-// Blocked right-looking Cholesky: kCholB columns per step and two team
-// barriers per step (instead of one per column), so the trailing triangle is
-// read and rewritten once per kCholB columns.  The result has the layout of
-// the column-by-column version: the pivot d_k on the diagonal (+inf for a
-// dependent row), L below it.
-//   Step at column k0, block b = min(kCholB, m - k0):
-//   1. every CTA factors the diagonal block D = M[k0.., k0..] (b x b) in
-//      shared memory, column by column with the pivot rule above, so every
-//      CTA takes the same decisions without communicating; CTA 0 writes it
-//      back;
-//   2. every row i below the block is solved against it (warp per row):
-//      L_ik = (M_ik - sum_{t<k} L_it L_kt) s_k with s_k = 1/sqrt(d_k) (0 for
-//      a dependent row);
-//   -- team barrier --
-//   3. the trailing lower triangle is updated by the panel (warp per row i,
-//      lanes over the columns j <= i): M_ij -= sum_t L_it L_jt.
-//   -- team barrier --
-// Returns false (in every thread of the team) only for a pivot that is
-// negative beyond rounding or not a number.
+// Blocked factorisation M = L L' and X = L^{-1} in one sweep, one team barrier
+// per kCholB columns: X is the right half of [M | I] under the same
+// elimination, so its updates are products of the same shape as those of the
+// trailing triangle and share their barriers and their load balance.
+//   The step at column k1 (the block before it, at k0 = k1 - kCholB, is final:
+//   L[k1.., k0..k1) and X[k0..k1, 0..k1)):
+//   A. every CTA updates the diagonal block D = M[k1.., k1..] with L, factors
+//      it with the pivot rule above and inverts its factor, in shared memory
+//      (every CTA takes the same decisions without communicating);
+//   B. the block's column of L below it, L_iq = (M_iq - L_ip L_qp') D^{-1}', in
+//      units of 32 rows, and its row of X, X_q = D^{-1} (X_q - L_qp X_p), in
+//      units of 32 columns;
+//   C. the rest, M_ij -= L_ip L_jp' and X_ij -= L_ip X_pj, in 32 x 32 tiles.
+//   The units of B and C are dealt to the team's CTAs in turn; the operands of
+//   the next unit are loaded into registers while one is computed.
+// The FP64 pipe bounds B and C (2 multiply-adds per clock per SM: a 32 x 32 x 16
+// tile is 4 us, its loads 1.5); blocks of 16 columns keep A, the serial part
+// (about 6 us), and the padding of small m low.  Measured, factor and inverse:
+// m = 2000 66 -> 9.6 ms, m = 200 2.1 -> 0.41 ms (before: a warp per row or column
+// with one dependent sum each, two barriers per 16 columns, and the columns of
+// the inverse by forward substitution).
 constexpr int kCholB = 16;
+constexpr int kTile = 32;
 
-template <typename T>
-__device__ __noinline__ bool dense_chol_panel(double* M, int m, int k0, const T* jinv) {
-    __shared__ double D[kCholB][kCholB];
-    __shared__ double sc[kCholB];
-    __shared__ int bad;
-    const int b = min(kCholB, m - k0);
-    for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-        const int r = e / b, c = e % b;
-        D[r][c] = r >= c ? __ldcg(M + (size_t)(k0 + r) * m + k0 + c) : 0.0;
+struct DenseShared {
+    double A[kTile][kCholB + 1];       // L_ip rows of a unit (B: then the unit's block)
+    double B[kTile][kCholB + 1];       // L_jp rows (tiles of M), or
+                                       // X_p columns, B[j][t] = X[k0 + t][j0 + j]
+    double Lq[kCholB][kCholB + 1];     // L[k1.., k0..]
+    double D[kCholB][kCholB + 1];      // diagonal block, then its factor
+    double Di[kCholB][kCholB + 1];     // inverse of the factor (row 0 for a dependent row)
+    int bad;
+};
+__device__ __forceinline__ DenseShared& dense_smem() {
+    __shared__ DenseShared s;
+    return s;
+}
+
+// Part A's serial piece, one warp: lane r (mod 16) holds row r of D.  L D L'
+// without square roots on the way (a quotient per column), scaled by 1/sqrt(d)
+// at the end, then the inverse factor, lane c its column c.
+static __device__ __noinline__ void dense_diag(double tau_lane) {
+    DenseShared& S = dense_smem();
+    const int lane = threadIdx.x & 31, r = lane & (kCholB - 1);
+    constexpr unsigned full = 0xffffffffu;
+    double a[kCholB];
+#pragma unroll
+    for (int c = 0; c < kCholB; ++c) a[c] = S.D[r][c];
+    bool fail = false, dep_own = false;
+    double d_own = 1.0;
+#pragma unroll
+    for (int k = 0; k < kCholB; ++k) {
+        const double d = __shfl_sync(full, a[k], k), tau = __shfl_sync(full, tau_lane, k);
+        fail = fail || d != d || d < -1e3 * tau;
+        const bool dep = !(d > tau) || d == INFINITY;
+        if (r == k) {
+            dep_own = dep;
+            d_own = d;
+        }
+        const double v = dep ? 0.0 : a[k] * __drcp_rn(d);
+#pragma unroll
+        for (int j = k + 1; j < kCholB; ++j) a[j] = fma(-v, __shfl_sync(full, a[k], j), a[j]);
     }
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
-    if (threadIdx.x < 32) {                              // one warp factors the block
-        const int lane = threadIdx.x;
-        for (int k = 0; k < b; ++k) {
-            const double d = D[k][k];
-            const double tau = 1e-13 / (double)__ldcg(jinv + k0 + k);
-            const bool fail = d != d || d < -1e3 * tau;
-            const bool dep = !(d > tau) || d == INFINITY;
-            const double s = dep ? 0.0 : 1.0 / sqrt(d);
-            __syncwarp();
-            if (lane == 0) {
-                if (fail) bad = 1;
-                sc[k] = s;
-                D[k][k] = dep ? INFINITY : d;
+    const double s_own = dep_own ? 0.0 : 1.0 / sqrt(d_own);
+#pragma unroll
+    for (int k = 0; k < kCholB; ++k) {
+        const double s = __shfl_sync(full, s_own, k);
+        if (lane < kCholB) S.D[r][k] = r > k ? a[k] * s : 0.0;   // strictly lower part of L
+    }
+    __syncwarp();
+    double x[kCholB];
+#pragma unroll
+    for (int i = 0; i < kCholB; ++i) x[i] = i == r ? 1.0 : 0.0;
+#pragma unroll
+    for (int t = 0; t < kCholB; ++t) {
+        x[t] *= __shfl_sync(full, s_own, t);
+#pragma unroll
+        for (int i = t + 1; i < kCholB; ++i) x[i] = fma(-S.D[i][t], x[t], x[i]);
+    }
+    if (lane < kCholB) {
+#pragma unroll
+        for (int i = 0; i < kCholB; ++i) S.Di[i][r] = i >= r ? x[i] : 0.0;
+    }
+    if (lane == 0) S.bad = fail ? 1 : 0;
+    __syncwarp();
+}
+
+// What a unit of B or C works on.
+struct DenseUnit {
+    int kind;          // 0: panel rows, 1: row of X, 2: tile of M, 3: tile of X
+    int i0, j0;        // first row and column of its block
+};
+
+// The units of the step at k1, numbered from 0: nB1 of kind 0, nB2 of kind 1,
+// then the tiles of X (nt rows of nX) and of M (lower triangle of nt).
+struct DensePlan {
+    int k0, k1, k2, nB1, nB2, nX;
+    long long total;
+};
+__device__ __forceinline__ DensePlan dense_plan(int m, int k1) {
+    DensePlan P;
+    P.k1 = k1;
+    P.k0 = k1 - kCholB;                                  // < 0: no block before
+    P.k2 = min(m, k1 + kCholB);
+    const int nt = (m - P.k2 + kTile - 1) / kTile;
+    P.nB1 = nt;
+    P.nX = k1 > 0 ? (k1 + kTile - 1) / kTile : 0;
+    P.nB2 = P.nX;
+    P.total = (long long)P.nB1 + P.nB2 + (k1 > 0 ? (long long)nt * P.nX + (long long)nt * (nt + 1) / 2 : 0);
+    return P;
+}
+__device__ __forceinline__ DenseUnit dense_unit(const DensePlan& P, long long u) {
+    DenseUnit U;
+    if (u < P.nB1) {
+        U.kind = 0;
+        U.i0 = P.k2 + (int)u * kTile;
+        U.j0 = P.k1;
+        return U;
+    }
+    u -= P.nB1;
+    if (u < P.nB2) {
+        U.kind = 1;
+        U.i0 = P.k1;
+        U.j0 = (int)u * kTile;
+        return U;
+    }
+    u -= P.nB2;
+    const long long tx = (long long)P.nB1 * P.nX;
+    if (u < tx) {
+        U.kind = 3;
+        U.i0 = P.k2 + (int)(u / P.nX) * kTile;
+        U.j0 = (int)(u % P.nX) * kTile;
+        return U;
+    }
+    u -= tx;
+    int bi = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+    while ((long long)(bi + 1) * (bi + 2) / 2 <= u) ++bi;
+    while ((long long)bi * (bi + 1) / 2 > u) --bi;
+    U.kind = 2;
+    U.i0 = P.k2 + bi * kTile;
+    U.j0 = P.k2 + (int)(u - (long long)bi * (bi + 1) / 2) * kTile;
+    return U;
+}
+
+// Registers of one unit: R = 1024 / threads elements of its block (rows ty, ty +
+// threads / 32, ...; column tx), and its share of the two operands.
+template <int R>
+struct DenseRegs {
+    double c[R], a[R], b[R];
+};
+
+template <int R>
+__device__ __forceinline__ void dense_load(const double* M, const double* X, int m, const DensePlan& P,
+                                           const DenseUnit& U, DenseRegs<R>& G) {
+    constexpr int kRows = kTile / R;                     // rows covered by the threads at once
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int k0 = P.k0, k1 = P.k1;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int r = ty + q * kRows;
+        // the block: 32 x 32, or 32 rows x 16 (kind 0), or 16 rows x 32 (kind 1)
+        const int i = U.i0 + r, j = U.j0 + tx;
+        double c = 0.0;
+        if (U.kind == 0) { if (tx < kCholB && i < m && j < m) c = __ldcg(M + (size_t)i * m + j); }
+        else if (U.kind == 1) { if (r < kCholB && i < m && j < k0) c = __ldcg(X + (size_t)i * m + j); }
+        else if (U.kind == 2) { if (i < m && j <= i) c = __ldcg(M + (size_t)i * m + j); }
+        else { if (i < m && j < k0) c = __ldcg(X + (size_t)i * m + j); }   // block column k0: first update
+        G.c[q] = c;
+        // the operands: L[i0 + row, k0 + t] by (row = r, t = tx) for tx < 16; the
+        // other half of the lanes loads L[j0 + row, k0 + t] (kind 2); kinds 1
+        // and 3: X[k0 + t, j0 + tx] by (t = r) for r < 16
+        double a = 0.0, b = 0.0;
+        if (k0 >= 0) {
+            const int t = tx & (kCholB - 1);
+            if (tx < kCholB) {
+                if (U.kind != 1 && i < m) a = __ldcg(M + (size_t)i * m + k0 + t);
+            } else if (U.kind == 2) {
+                if (U.j0 + r < m) a = __ldcg(M + (size_t)(U.j0 + r) * m + k0 + t);
             }
-            if (lane > k && lane < b) D[lane][k] *= s;  // column k of L in the block
-            __syncwarp();
-            for (int i = k + 1 + lane; i < b; i += 32)   // rows below: update columns k+1 .. i
-                for (int j = k + 1; j <= i; ++j) D[i][j] = fma(-D[i][k], D[j][k], D[i][j]);
-            __syncwarp();
+            if ((U.kind == 1 || U.kind == 3) && r < kCholB && j < k1) b = __ldcg(X + (size_t)(k0 + r) * m + j);
         }
+        G.a[q] = a;
+        G.b[q] = b;
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void dense_compute(double* M, double* X, int m, const DensePlan& P, const DenseUnit& U,
+                                              const DenseRegs<R>& G) {
+    DenseShared& S = dense_smem();
+    constexpr int kRows = kTile / R;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    double acc[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) acc[q] = G.c[q];
+    if (P.k0 >= 0) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int r = ty + q * kRows, t = tx & (kCholB - 1);
+            if (tx < kCholB) S.A[r][t] = G.a[q];
+            else if (U.kind == 2) S.B[r][t] = G.a[q];
+            if ((U.kind == 1 || U.kind == 3) && r < kCholB) S.B[tx][r] = G.b[q];
+        }
+        __syncthreads();
+        if (U.kind == 0) {                               // columns of the block: rows of L_q
+            if (tx < kCholB)
+#pragma unroll
+                for (int t = 0; t < kCholB; ++t) {
+                    const double y = S.Lq[tx][t];
+#pragma unroll
+                    for (int q = 0; q < R; ++q) acc[q] = fma(-S.A[ty + q * kRows][t], y, acc[q]);
+                }
+        } else if (U.kind == 1) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                if (ty + q * kRows < kCholB)
+#pragma unroll
+                    for (int t = 0; t < kCholB; ++t) acc[q] = fma(-S.Lq[ty + q * kRows][t], S.B[tx][t], acc[q]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < kCholB; ++t) {
+                const double y = S.B[tx][t];
+#pragma unroll
+                for (int q = 0; q < R; ++q) acc[q] = fma(-S.A[ty + q * kRows][t], y, acc[q]);
+            }
+        }
+        __syncthreads();
+    }
+    if (U.kind >= 2) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int i = U.i0 + ty + q * kRows, j = U.j0 + tx;
+            if (U.kind == 2) { if (i < m && j <= i) M[(size_t)i * m + j] = acc[q]; }
+            else { if (i < m && j < P.k1) X[(size_t)i * m + j] = acc[q]; }
+        }
+        return;
+    }
+    // kinds 0 and 1: the block through shared memory, times the inverse factor
+    if (U.kind == 0) {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            if (tx < kCholB) S.A[ty + q * kRows][tx] = acc[q];
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[q] = 0.0;
+        if (tx < kCholB)
+#pragma unroll
+            for (int t = 0; t < kCholB; ++t) {
+                const double y = S.Di[tx][t];
+#pragma unroll
+                for (int q = 0; q < R; ++q) acc[q] = fma(S.A[ty + q * kRows][t], y, acc[q]);
+            }
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int i = U.i0 + ty + q * kRows, j = U.j0 + tx;
+            if (tx < kCholB && i < m && j < m) M[(size_t)i * m + j] = acc[q];
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+            if (ty + q * kRows < kCholB) S.B[tx][ty + q * kRows] = acc[q];
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int r = ty + q * kRows;
+            if (r < kCholB) {
+                double x = 0.0;
+#pragma unroll
+                for (int t = 0; t < kCholB; ++t) x = fma(S.Di[r][t], S.B[tx][t], x);
+                const int i = U.i0 + r, j = U.j0 + tx;
+                if (i < m && j < P.k1) X[(size_t)i * m + j] = x;
+            }
+        }
+    }
+    __syncthreads();                                     // the operands of the next unit may be stored
+}
+
+template <int R>
+__device__ __noinline__ void dense_units(double* M, double* X, int m, int k1) {
+    const DensePlan P = dense_plan(m, k1);
+    const int size = team_size();
+    long long u = team_rank();
+    if (u >= P.total) return;                            // CTA-uniform
+    DenseUnit U = dense_unit(P, u);
+    DenseRegs<R> G;
+    dense_load<R>(M, X, m, P, U, G);
+    while (true) {
+        const long long un = u + size;
+        DenseUnit V = U;
+        DenseRegs<R> H = G;
+        if (un < P.total) {
+            V = dense_unit(P, un);
+            dense_load<R>(M, X, m, P, V, H);
+        }
+        dense_compute<R>(M, X, m, P, U, G);
+        if (un >= P.total) break;
+        u = un;
+        U = V;
+        G = H;
+    }
+}
+
+// The step at column k1 (0, kCholB, 2 kCholB, ...).  Returns false (in every
+// thread of the team) only for a pivot that is negative beyond rounding or not
+// a number.
+template <typename T>
+__device__ __noinline__ bool dense_factor_step(double* M, double* X, int m, int k1, const T* jinv) {
+    DenseShared& S = dense_smem();
+    const int k0 = k1 - kCholB;
+    __syncthreads();                                     // the shared blocks are free
+    for (int e = threadIdx.x; e < kCholB * kCholB; e += blockDim.x) {
+        const int r = e / kCholB, c = e % kCholB;
+        double d = r == c ? 1.0 : 0.0, l = 0.0;          // rows past m: the identity
+        if (k1 + r < m) {
+            if (c <= r) d = __ldcg(M + (size_t)(k1 + r) * m + k1 + c);
+            if (k0 >= 0) l = __ldcg(M + (size_t)(k1 + r) * m + k0 + c);
+        }
+        S.D[r][c] = d;
+        S.Lq[r][c] = l;
+    }
+    double tau = 0.0;
+    if (threadIdx.x < 32) {
+        const int r = threadIdx.x & (kCholB - 1);
+        tau = k1 + r < m ? 1e-13 / (double)__ldcg(jinv + k1 + r) : 0.0;
     }
     __syncthreads();
-    if (bad) return false;                               // CTA-uniform (and team-uniform: same data)
-    if (team_rank() == 0)
-        for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-            const int r = e / b, c = e % b;
-            if (r >= c) M[(size_t)(k0 + r) * m + k0 + c] = D[r][c];
+    if (k0 >= 0)
+        for (int e = threadIdx.x; e < kCholB * kCholB; e += blockDim.x) {
+            const int r = e / kCholB, c = e % kCholB;
+            double d = S.D[r][c];
+            if (c <= r) {
+#pragma unroll
+                for (int t = 0; t < kCholB; ++t) d = fma(-S.Lq[r][t], S.Lq[c][t], d);
+            }
+            S.D[r][c] = d;
         }
-    // panel rows below the block, warp per row, lane k holds L_ik
-    const int lane = threadIdx.x & 31;
-    for (int i = k0 + b + global_warp(); i < m; i += global_warps()) {
-        double* Mi = M + (size_t)i * m + k0;
-        double x = lane < b ? __ldcg(Mi + lane) : 0.0;
-        for (int k = 0; k < b; ++k) {
-            const double xk = __shfl_sync(0xffffffffu, x, k) * sc[k];   // final L_ik
-            if (lane == k) x = xk;
-            if (lane > k && lane < b) x = fma(-xk, D[lane][k], x);
+    __syncthreads();
+    if (threadIdx.x < 32) dense_diag(tau);
+    __syncthreads();
+    if (S.bad) return false;                             // CTA-uniform (and team-uniform: same data)
+    if (team_rank() == 0)                                // the diagonal block of X, its zeros too
+        for (int e = threadIdx.x; e < kCholB * kCholB; e += blockDim.x) {
+            const int r = e / kCholB, c = e % kCholB;
+            if (k1 + r < m && k1 + c < m) X[(size_t)(k1 + r) * m + k1 + c] = S.Di[r][c];
         }
-        if (lane < b) Mi[lane] = x;
-    }
+    if (blockDim.x == 1024) dense_units<1>(M, X, m, k1);
+    else if (blockDim.x == 512) dense_units<2>(M, X, m, k1);
+    else dense_units<4>(M, X, m, k1);
     return true;
 }
 
-// Step 3 of the blocked factorisation: M_ij -= sum_t L_it L_jt for
-// k0 + b <= j <= i < m, with L the panel just written.
-static __device__ __noinline__ void dense_chol_trailing(double* M, int m, int k0) {
-    const int b = min(kCholB, m - k0);
-    const int lane = threadIdx.x & 31;
-    for (int i = k0 + b + global_warp(); i < m; i += global_warps()) {
-        const double* Li = M + (size_t)i * m + k0;
-        double li[kCholB];
-#pragma unroll
-        for (int t = 0; t < kCholB; ++t) li[t] = t < b ? __ldcg(Li + t) : 0.0;
-        double* Mi = M + (size_t)i * m;
-        for (int j = k0 + b + lane; j <= i; j += 32) {
-            const double* Lj = M + (size_t)j * m + k0;
-            double acc = 0.0;
-#pragma unroll
-            for (int t = 0; t < kCholB; ++t)
-                if (t < b) acc = fma(li[t], __ldcg(Lj + t), acc);
-            Mi[j] -= acc;
-        }
+// dM <- X' (upper triangle, row-major), 32 x 32 tiles through shared memory.
+static __device__ __noinline__ void dense_transpose(const double* X, double* Mt, int m) {
+    DenseShared& S = dense_smem();
+    double(*tile)[kTile + 1] = reinterpret_cast<double(*)[kTile + 1]>(&S);   // 8.4 KB of its 13
+    const int nt = (m + kTile - 1) / kTile;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (long long u = team_rank(); u < (long long)nt * nt; u += team_size()) {
+        const int i0 = (int)(u / nt) * kTile, j0 = (int)(u % nt) * kTile;
+        if (j0 > i0) continue;                           // CTA-uniform
+        __syncthreads();
+        for (int r = ty; r < kTile; r += nw)
+            tile[r][tx] = (i0 + r < m && j0 + tx <= i0 + r) ? __ldcg(X + (size_t)(i0 + r) * m + j0 + tx) : 0.0;
+        __syncthreads();
+        for (int r = ty; r < kTile; r += nw)
+            if (j0 + r < m && i0 + tx < m && i0 + tx >= j0 + r) Mt[(size_t)(j0 + r) * m + i0 + tx] = tile[tx][r];
     }
 }
 
-// X = L^{-1} (column-major) by forward substitution, warp per column c:
-// x_i = (delta_ic - sum_{c <= t < i} L_it x_t) / L_ii for i >= c, with
-// L_ii = sqrt(d_i) from the pivot kept on the diagonal.
-template <typename T>
-__device__ __noinline__ void phase_dense_inverse(const IterParams<T>& P) {
-    const double* M = sync_smem().dM;
-    double* X = sync_smem().dX;
-    const int m = P.m;
+// Rows of a triangular m x m matrix times a vector: out(i, sum_j T_ij v_j), j in
+// [0, i] (lower) or [i, m) (upper).  A warp takes R consecutive rows at a time,
+// so that their sums over the lanes are taken together (9 additions a lane for
+// eight rows instead of 40) and R loads of the matrix per element of v are in
+// flight; consecutive groups go to different CTAs.  The FP64 pipe bounds the
+// small teams, latency the whole grid (R = 1 there).  Measured, both products:
+// m = 2000 on 152 CTAs 429 -> 19 us, m = 200 31 -> 6.8 us (before: a thread per
+// row of X, a warp per column of it).
+template <int R, bool kUpper, typename Tv, typename Out>
+__device__ __forceinline__ void tri_rows(const double* T, int m, const Tv* v, const Out& out) {
     const int lane = threadIdx.x & 31;
-    for (int c = global_warp(); c < m; c += global_warps()) {
-        double* Xc = X + (size_t)c * m;
-        for (int i = c; i < m; ++i) {
-            const double* Li = M + (size_t)i * m;
-            double acc = 0.0;
-            for (int t = c + lane; t < i; t += 32) acc = fma(__ldcg(Li + t), Xc[t], acc);
-            acc = warp_sum(acc);
-            const double xi = ((i == c ? 1.0 : 0.0) - acc) / sqrt(__ldcg(Li + i));
-            if (lane == 0) Xc[i] = xi;
-            __syncwarp();
+    const int size = team_size(), nw = (int)(blockDim.x >> 5) * size;
+    const int w = (int)(threadIdx.x >> 5) * size + team_rank();
+    const int ng = (m + R - 1) / R;
+    constexpr int U = R == 1 ? 8 : R == 2 ? 4 : 1;
+    for (int g = w; g < ng; g += nw) {
+        // the long rows first: they are the last ones (lower) or the first
+        const int i0 = (kUpper ? g : ng - 1 - g) * R;
+        const int lo = kUpper ? (i0 & ~31) : 0, hi = kUpper ? m : min(m, i0 + R);
+        double a[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r] = 0.0;
+        for (int j0 = lo + lane; j0 < hi; j0 += 32 * U) {
+            double x[U], t[U][R];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int j = j0 + 32 * u;
+                x[u] = j < hi ? (double)__ldcg(v + j) : 0.0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int i = i0 + r;
+                    const bool in = i < m && j < hi && (kUpper ? j >= i : j <= i);
+                    t[u][r] = in ? __ldcg(T + (size_t)i * m + j) : 0.0;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int r = 0; r < R; ++r) a[r] = fma(t[u][r], x[u], a[r]);
         }
+        warp_sums<R>(a);
+        const int i = i0 + warp_sums_index<R>(lane);
+        if ((lane & (32 / R - 1)) == 0 && i < m) out(i, a[0]);
     }
 }
+template <bool kUpper, typename Tv, typename Out>
+__device__ __forceinline__ void tri_product(const double* T, int m, const Tv* v, const Out& out) {
+    const int per_warp = m / (int)(team_size() * (blockDim.x >> 5));   // rows a warp has
+    if (per_warp >= 8) tri_rows<8, kUpper>(T, m, v, out);
+    else if (per_warp >= 2) tri_rows<2, kUpper>(T, m, v, out);
+    else tri_rows<1, kUpper>(T, m, v, out);
+}
 
-// y = X r0 (r0 = the FP64 residual of the projection system, in V.r), thread
-// per row; y is kept in V.p (unused by the dense path).
+// y = X r0 (r0 = the FP64 residual of the projection system, in V.r); y is
+// kept in V.p (unused by the dense path).
 template <typename T>
 __device__ __noinline__ void phase_dense_y(const IterParams<T>& P) {
-    const double* X = sync_smem().dX;
-    const int m = P.m;
-    const T* r = P.V.r;
-    for (int i = global_tid(); i < m; i += global_threads()) {
-        // four independent partial sums keep four loads of X in flight
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        int c = 0;
-        for (; c + 3 <= i; c += 4) {
-            a0 = fma(__ldcg(X + (size_t)c * m + i), (double)__ldcg(r + c), a0);
-            a1 = fma(__ldcg(X + (size_t)(c + 1) * m + i), (double)__ldcg(r + c + 1), a1);
-            a2 = fma(__ldcg(X + (size_t)(c + 2) * m + i), (double)__ldcg(r + c + 2), a2);
-            a3 = fma(__ldcg(X + (size_t)(c + 3) * m + i), (double)__ldcg(r + c + 3), a3);
-        }
-        for (; c <= i; ++c) a0 = fma(__ldcg(X + (size_t)c * m + i), (double)__ldcg(r + c), a0);
-        P.V.p[i] = (T)((a0 + a1) + (a2 + a3));
-    }
+    tri_product<false>(sync_smem().dX, P.m, P.V.r, [&](int i, double y) { P.V.p[i] = (T)y; });
 }
 
-// w += X' y: warp per column c, x_c = sum_{i >= c} X_ic y_i.
+// w += X' y.
 template <typename T>
 __device__ __noinline__ void phase_dense_x(const IterParams<T>& P) {
-    const double* X = sync_smem().dX;
-    const int m = P.m;
-    const int lane = threadIdx.x & 31;
-    const T* y = P.V.p;
-    for (int c = global_warp(); c < m; c += global_warps()) {
-        const double* Xc = X + (size_t)c * m;
-        double a0 = 0.0, a1 = 0.0;
-        int i = c + lane;
-        for (; i + 32 < m; i += 64) {
-            a0 = fma(__ldcg(Xc + i), (double)__ldcg(y + i), a0);
-            a1 = fma(__ldcg(Xc + i + 32), (double)__ldcg(y + i + 32), a1);
-        }
-        if (i < m) a0 = fma(__ldcg(Xc + i), (double)__ldcg(y + i), a0);
-        const double acc = warp_sum(a0 + a1);
-        if (lane == 0) P.X.w[c] += acc;
-    }
+    tri_product<true>(sync_smem().dM, P.m, P.V.p, [&](int c, double x) { P.X.w[c] += x; });
 }
 
 // ---------------------------------------------------------------------------
@@ -2170,16 +2450,13 @@ static __device__ __noinline__ void polish_loop(const IterParams<double>& P, con
             phase_dense_assemble(P);
             if (!grid_sync(&P.ctl->err)) break;
             bool fine = true;
-            for (int k0 = 0; k0 < P.m; k0 += kCholB) {
-                if (!dense_chol_panel(sync_smem().dM, P.m, k0, P.V.jinv)) dense = false;
-                if (!(fine = grid_sync(&P.ctl->err))) break;
-                if (!dense) break;
-                dense_chol_trailing(sync_smem().dM, P.m, k0);
+            for (int k1 = 0; k1 < P.m && dense; k1 += kCholB) {
+                if (!dense_factor_step(sync_smem().dM, sync_smem().dX, P.m, k1, P.V.jinv)) dense = false;
                 if (!(fine = grid_sync(&P.ctl->err))) break;
             }
             if (!fine) break;
             if (dense) {
-                phase_dense_inverse(P);
+                dense_transpose(sync_smem().dX, sync_smem().dM, P.m);
                 if (!grid_sync(&P.ctl->err)) break;
                 used_dense = 1.0;
             }
@@ -2361,19 +2638,16 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                 factor_ok = false;
                 phase_dense_assemble(P);
                 ACS_SYNC(PH_DENSE_ASSEMBLE);
-                for (int k0 = 0; k0 < P.m && dense; k0 += kCholB) {
-                    if (!dense_chol_panel(sync_smem().dM, P.m, k0, P.V.jinv)) {
+                for (int k1 = 0; k1 < P.m && dense; k1 += kCholB) {
+                    if (!dense_factor_step(sync_smem().dM, sync_smem().dX, P.m, k1, P.V.jinv)) {
                         dense = false;
                         dense_failed = true;
                     }
                     ACS_SYNC(PH_DENSE_FACTOR);
-                    if (!dense) break;
-                    dense_chol_trailing(sync_smem().dM, P.m, k0);
-                    ACS_SYNC(PH_DENSE_FACTOR);
                 }
                 if (!ok) break;
                 if (dense) {
-                    phase_dense_inverse(P);
+                    dense_transpose(sync_smem().dX, sync_smem().dM, P.m);
                     ACS_SYNC(PH_DENSE_INVERSE);
                     ++nfactor;
                     factor_ok = true;
@@ -2399,7 +2673,7 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         bool trouble = false;                                   // FP32 solve cannot keep up
         if (dense) {
             // one exact correction: dw = X'(X r0)
-            phase_rhs(P);
+            phase_rhs_plain(P);
             ++nA64;
             ACS_SYNC(PH_RHS);
             phase_dense_y(P);
