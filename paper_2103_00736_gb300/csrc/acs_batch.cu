@@ -300,6 +300,7 @@ int prepare_members(Batch* B, int count, const acs_instance* members, int* bad) 
                     continue;
                 }
                 own[i].stored = (long long)own[i].H.A.col.size();
+                own[i].full = I.row_ptr[I.m] == (int64_t)I.m * I.n;
             }
         }
     });

@@ -576,6 +576,7 @@ int acs_problem_create(int32_t m, int32_t n, const int64_t* row_ptr, const int32
     rc |= cudaMemsetAsync(P->ctl, 0, sizeof(acs::Control), P->stream) != cudaSuccess;
     if (rc || cudaStreamSynchronize(P->stream) != cudaSuccess) { free_all(P); delete P; return ACS_ERR_CUDA; }
     if (P->grid32 > P->max_ctas || P->grid64 > P->max_ctas || P->grid32 > 256 || P->grid64 > 256) { free_all(P); delete P; return ACS_ERR_CUDA; }
+    P->small_ctas = acs::small_cluster(P);
     step("finish");
     P->create_h2d = P->h2d_bytes;
     P->create_d2h = P->d2h_bytes;

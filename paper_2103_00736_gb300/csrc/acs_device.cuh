@@ -54,13 +54,19 @@ __device__ __forceinline__ int ld_volatile_int(const int* p) { return *(volatile
 // the wait records ACS_ERR_DEVICE_TIMEOUT and grid_sync returns false in
 // every thread; the caller then leaves the kernel.
 constexpr int kMaxGrid = 256;   // CTAs of a persistent launch (one per SM)
+constexpr int kMaxCluster = 16; // CTAs of a launch that is one cluster
 
 // Scalars that steer the solve loop and the CG, computed once per CTA.
 struct CondRange {
     double alpha, lmin, lmax;
     bool any;
 };
+enum Count : int {
+    CT_A = 0, CT_AT, CT_A64, CT_AT64, CT_COND, CT_CHECK, CT_A32, CT_AT32, CT_DENSE, CT_FACTOR, CT_CG, CT_COUNT
+};
 struct LoopScalars {
+    long long count[CT_COUNT];   // passes of this loop (thread 0)
+    long long win_cg;            // CG iterations since the last rescaling (thread 0)
     double gam, gam_prev, alpha, alpha_prev, beta, thr;   // CG
     double floor_r, target, best, best_ref;               // polish solves
     double ds, snorm, eta, d0, d1;                        // step norms, inexactness factor
@@ -78,6 +84,7 @@ struct LoopScalars {
 };
 
 struct SyncShared {
+    int cluster;              // the team is one thread-block cluster (barriers in hardware)
     int team_rank;            // this CTA's rank in the team working on one problem
     int team_size;            // CTAs in the team (the whole grid for a single solve)
     unsigned long long* bar;  // the team's monotonic barrier arrival counter
@@ -88,6 +95,7 @@ struct SyncShared {
     double out[kMaxRed];      // grid-reduced values of the last barrier
     double wsum[kWarps][kMaxRed];   // the warps' contributions to the next one
     double gsum[kWarps][kMaxRed];   // the CTAs' contributions, by the warp that gathered them
+    double cslot[2][kMaxCluster][kMaxRed];   // a cluster's partials, written by its CTAs
     unsigned opmask;          // bit k: value k is combined by max (else by sum)
     int nv;                   // number of values reduced at the next barrier
     LoopScalars lp;           // scalars of the solve loop, written by warp 0 at the barriers
@@ -112,9 +120,10 @@ __device__ __forceinline__ SyncShared& sync_smem() {
 // single-problem launch, or a group of CTAs (often one) of a batched launch.
 // Phases index coordinates, rows and cones by the thread's rank in its team.
 __device__ __forceinline__ void team_set(int rank, int size, unsigned long long* bar, double* partials,
-                                         double* dense_M = nullptr, double* dense_X = nullptr) {
+                                         double* dense_M = nullptr, double* dense_X = nullptr, int cluster = 0) {
     SyncShared& S = sync_smem();
     if (threadIdx.x == 0) {
+        S.cluster = cluster;
         S.team_rank = rank;
         S.team_size = size;
         S.bar = bar;
@@ -131,6 +140,24 @@ __device__ __forceinline__ int global_tid() { return team_rank() * (int)blockDim
 __device__ __forceinline__ int global_threads() { return team_size() * (int)blockDim.x; }
 __device__ __forceinline__ int global_warp() { return global_tid() >> 5; }
 __device__ __forceinline__ int global_warps() { return global_threads() >> 5; }
+
+// The parameter block of a solve, copied to shared memory once per launch or
+// member.  The phases take it by reference, so each field they use is a load
+// through a generic address; from a kernel's parameters or from global memory
+// that load misses L1 after every barrier (the barrier's acquire empties it), an
+// L2 round trip before the first useful load of a phase and again for each
+// pointer the compiler cannot keep in a register.  Measured: 0.5 to 1.2 us of every
+// phase (the CG passes of a 1000 x 5000 LP 3.4 -> 3.0 and 6.6 -> 6.2 us).
+template <typename T, int kWhich = 0>
+__device__ __forceinline__ const IterParams<T>& stage_params(const IterParams<T>& P) {
+    static_assert(sizeof(IterParams<T>) % 8 == 0, "copied by 8-byte words");
+    __shared__ __align__(16) unsigned long long buf[sizeof(IterParams<T>) / 8];
+    __syncthreads();                                     // no one reads an earlier block any more
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(&P);
+    for (int i = threadIdx.x; i < (int)(sizeof(IterParams<T>) / 8); i += blockDim.x) buf[i] = src[i];
+    __syncthreads();
+    return *reinterpret_cast<const IterParams<T>*>(buf);
+}
 
 __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll
@@ -317,6 +344,19 @@ __device__ __forceinline__ bool gather_slots(const double* part, unsigned long l
     return ok;
 }
 
+// Barrier of all threads of the cluster; what any of them wrote before it is
+// visible to all after it.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// v to the same variable of CTA `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(double* var, int rank, double v) {
+    unsigned local = (unsigned)__cvta_generic_to_shared(var), remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+}
+
 // The barrier up to the reduced values.
 //
 // Without values, thread 0 adds 1 to the team's monotonic arrival counter
@@ -329,17 +369,32 @@ __device__ __forceinline__ bool gather_slots(const double* part, unsigned long l
 // news that that CTA has arrived, so that one L2 round trip after the last
 // arrival every CTA has every partial (counter, then partials: two).  The
 // counter is kept in step for the barriers without values.
-// A team of one CTA needs neither.  The caller follows with a CTA barrier.
+//
+// The error word is read while the wait is under way, so an error recorded
+// just before a barrier may be seen one barrier later; the CTA that recorded it
+// has left by then, and the others' next wait ends on the error word.
+//
+// A team that is one cluster uses the hardware's cluster barrier (which counts
+// threads that have not exited, so it cannot wait for a CTA that has left) and
+// exchanges partials through distributed shared memory.  A team of one CTA
+// needs neither.  The caller follows with a CTA barrier.
 static __device__ __noinline__ void grid_reduce(int* err) {
     SyncShared& S = sync_smem();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool cluster = S.cluster != 0;
     __syncthreads();                                   // the phase's writes and S.wsum are complete
     const unsigned target = S.gen + 1u;
     const int nv = S.nv;
     const int size = S.team_size;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (nv == 0 && cluster) {
+        cluster_sync();
+        if (threadIdx.x == 0) S.gen = target;
+        return;
+    }
     if (nv == 0) {
         if (threadIdx.x == 0) {
             bool fail = false;
+            const int e = ld_volatile_int(err);
             if (size > 1) {
                 red_add_release(S.bar, 1ull);
                 const unsigned long long want = (unsigned long long)target * size;
@@ -347,13 +402,15 @@ static __device__ __noinline__ void grid_reduce(int* err) {
                 for (int tries = 0; ld_acquire64(S.bar) < want; ++tries)
                     if (wait_expired(tries, t0, err)) { fail = true; break; }
             }
-            if (fail || ld_volatile_int(err) != 0) S.fail = 1;
+            if (fail || e != 0) S.fail = 1;
             S.gen = target;
         }
         return;
     }
     const unsigned opmask = S.opmask;
+    int e = 0;
     if (warp == 0) {
+        if (lane == 0) e = ld_volatile_int(err);
         const int nw = (int)(blockDim.x >> 5);
         double x[kMaxRed];
 #pragma unroll
@@ -365,7 +422,7 @@ static __device__ __noinline__ void grid_reduce(int* err) {
         if (size == 1) {
             // the error word is still checked so that a failed problem stops
             if (lane == 0) {
-                if (ld_volatile_int(err) != 0) S.fail = 1;
+                if (e != 0) S.fail = 1;
                 S.gen = target;
                 S.nv = 0;
             }
@@ -374,6 +431,28 @@ static __device__ __noinline__ void grid_reduce(int* err) {
         }
     }
     if (size == 1) return;
+    if (cluster) {
+        if (warp == 0 && lane < size)
+            for (int k = 0; k < nv; ++k) st_cluster(&S.cslot[target & 1u][S.team_rank][k], lane, S.out[k]);
+        cluster_sync();
+        if (warp == 0) {
+            double x[kMaxRed];
+#pragma unroll
+            for (int k = 0; k < kMaxRed; ++k) {
+                x[k] = 0.0;
+                if (k < nv)
+                    x[k] = lane < size ? S.cslot[target & 1u][lane][k] : ((opmask >> k) & 1u ? -INFINITY : 0.0);
+            }
+            warp_combine(x, nv, opmask, S.out);
+            if (lane == 0) {
+                if (e != 0) S.fail = 1;
+                S.gen = target;
+                S.nv = 0;
+            }
+            __syncwarp();
+        }
+        return;
+    }
     double* part = S.tpart + (target & 1u) * (2 * kMaxRed);
     if (warp == 0) {
         fence_gpu();                                    // the phase's writes come before the arrival
@@ -405,7 +484,7 @@ static __device__ __noinline__ void grid_reduce(int* err) {
             S.out[lane] = x;
         }
         if (lane == 0) {
-            if (ld_volatile_int(err) != 0) S.fail = 1;
+            if (e != 0) S.fail = 1;
             S.gen = target;
             S.nv = 0;
         }
@@ -1627,79 +1706,8 @@ __device__ __noinline__ void phase_kkt(const IterParams<T>& P) {
 // M = A O^2 A' (lower triangle), from row i of A and the columns of A it
 // touches (rows of A'): M_ik = sum_j O_j^2 a_ij a_kj.  Warp per row i, the
 // lanes over the entries of one column j at a time, in a fixed order.
-// Entry j of row i of a matrix whose rows are full (every column present,
-// in order), from its sliced-ELLPACK image: slice i / (32/g), lane group
-// i % (32/g), chunk j / g.
-__device__ __forceinline__ double sell_full_entry(const SellMat& A, int i, int j) {
-    const int g = A.g, h = 32 / g;
-    return __ldg(A.v64 + __ldg(A.sptr + i / h) + 32 * (j / g) + (i % h) * g + (j % g));
-}
-
-// M = A O^2 A' for full rows (the dense workloads): 64 x 64 tiles of the lower
-// triangle dealt to the team's CTAs, each the sum over j in increasing order
-// of 64 x 8 slabs of its two row blocks staged in shared memory (the first
-// scaled by O_j^2); thread (ty, tx) of the 32 x 32 threads owns rows
-// {ty, ty + 32} and columns {tx, tx + 32} of the tile.  FP64 throughout (the
-// FP64 pipe bounds it: about two FP64 multiply-adds per clock per SM here, so
-// the slabs stay small and leave L1 its carve-out).
-constexpr int kSyrkT = 64, kSyrkK = 8;
-
 template <typename T>
-__device__ __noinline__ void phase_dense_syrk(const IterParams<T>& P) {
-    __shared__ double Ai[kSyrkT][kSyrkK + 1];
-    __shared__ double Ak[kSyrkT][kSyrkK + 1];
-    double* M = sync_smem().dM;
-    const int m = P.m, n = P.n;
-    const int mt = (m + kSyrkT - 1) / kSyrkT;
-    const long long ntile = (long long)mt * (mt + 1) / 2;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (long long t = team_rank(); t < ntile; t += team_size()) {
-        // lower-triangular tile (bi, bk), bk <= bi, t = bi (bi + 1) / 2 + bk
-        int bi = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-        while ((long long)(bi + 1) * (bi + 2) / 2 <= t) ++bi;
-        while ((long long)bi * (bi + 1) / 2 > t) --bi;
-        const int bk = (int)(t - (long long)bi * (bi + 1) / 2);
-        const int i0 = bi * kSyrkT, k0 = bk * kSyrkT;
-        double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
-        for (int j0 = 0; j0 < n; j0 += kSyrkK) {
-            for (int e = threadIdx.x; e < kSyrkT * kSyrkK; e += blockDim.x) {
-                const int r = e / kSyrkK, c = e % kSyrkK, j = j0 + c;
-                double vi = 0.0, vk = 0.0;
-                if (j < n) {
-                    const double o = P.X.O[j];
-                    if (i0 + r < m) vi = sell_full_entry(P.A, i0 + r, j) * (o * o);
-                    if (k0 + r < m) vk = sell_full_entry(P.A, k0 + r, j);
-                }
-                Ai[r][c] = vi;
-                Ak[r][c] = vk;
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int c = 0; c < kSyrkK; ++c) {
-                const double x0 = Ai[ty][c], x1 = Ai[ty + 32][c];
-                const double y0 = Ak[tx][c], y1 = Ak[tx + 32][c];
-                a00 = fma(x0, y0, a00);
-                a01 = fma(x0, y1, a01);
-                a10 = fma(x1, y0, a10);
-                a11 = fma(x1, y1, a11);
-            }
-            __syncthreads();
-        }
-        const double acc[2][2] = {{a00, a01}, {a10, a11}};
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b) {
-                const int i = i0 + ty + 32 * a, k = k0 + tx + 32 * b;
-                if (i < m && k <= i) M[(size_t)i * m + k] = acc[a][b];
-            }
-    }
-}
-
-template <typename T>
-__device__ __noinline__ void phase_dense_assemble(const IterParams<T>& P) {
-    if (P.full_rows && blockDim.x == 1024) {            // dense rows: tiled product
-        phase_dense_syrk(P);
-        return;
-    }
+__device__ __noinline__ void phase_dense_scatter(const IterParams<T>& P) {
     double* M = sync_smem().dM;
     const int m = P.m;
     const int lane = threadIdx.x & 31;
@@ -2091,6 +2099,79 @@ __device__ __noinline__ bool dense_factor_step(double* M, double* X, int m, int 
     else if (blockDim.x == 512) dense_units<2>(M, X, m, k1);
     else dense_units<4>(M, X, m, k1);
     return true;
+}
+
+// M = A O^2 A' for full rows (the dense workloads): 32 x 32 tiles of the lower
+// triangle dealt to the team's CTAs, each the sum over j in increasing order of
+// 32 x 16 slabs of its two row blocks staged in shared memory (the first scaled
+// by O_j^2), the next slab's entries loaded while one is multiplied.  FP64
+// throughout; the FP64 pipe bounds it (a slab is 4 us), so the tiles are kept
+// small: n = 200, m = 160 has 15 of them.  Measured: m = 160, n = 200 on 16 CTAs
+// 65 us (233 on the grid before), m = 800, n = 1000 1.14 -> 0.90 ms (before: 64
+// x 64 tiles, 1024-thread CTAs only, without the prefetch).
+template <int R, typename T>
+__device__ __forceinline__ void dense_syrk(const IterParams<T>& P) {
+    DenseShared& S = dense_smem();
+    double* M = sync_smem().dM;
+    constexpr int kRows = kTile / R;
+    const int m = P.m, n = P.n;
+    const int nt = (m + kTile - 1) / kTile;
+    const long long ntile = (long long)nt * (nt + 1) / 2;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int t = tx & (kCholB - 1);
+    const SellMat& A = P.A;
+    const int g = A.g, h = 32 / g;
+    for (long long u = team_rank(); u < ntile; u += team_size()) {
+        int bi = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+        while ((long long)(bi + 1) * (bi + 2) / 2 <= u) ++bi;
+        while ((long long)bi * (bi + 1) / 2 > u) --bi;
+        const int i0 = bi * kTile, k0 = (int)(u - (long long)bi * (bi + 1) / 2) * kTile;
+        // the lower half of the lanes loads the rows of block i0, the upper half
+        // those of k0; entry j of a full row: slice row / h, chunk j / g
+        const double* row[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int i = (tx < kCholB ? i0 : k0) + ty + q * kRows;
+            row[q] = i < m ? A.v64 + __ldg(A.sptr + i / h) + (i % h) * g : nullptr;
+        }
+        double v[R], acc[R];
+        auto load = [&](int j) {
+            const double o = j < n && tx < kCholB ? P.X.O[j] : 1.0;
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                v[q] = j < n && row[q] ? __ldg(row[q] + 32 * (j / g) + (j % g)) * (o * o) : 0.0;
+        };
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[q] = 0.0;
+        load(t);
+        for (int j0 = 0; j0 < n; j0 += kCholB) {
+            __syncthreads();                             // the previous slab is used up
+#pragma unroll
+            for (int q = 0; q < R; ++q) (tx < kCholB ? S.A : S.B)[ty + q * kRows][t] = v[q];
+            __syncthreads();
+            if (j0 + kCholB < n) load(j0 + kCholB + t);
+#pragma unroll
+            for (int c = 0; c < kCholB; ++c) {
+                const double y = S.B[tx][c];
+#pragma unroll
+                for (int q = 0; q < R; ++q) acc[q] = fma(S.A[ty + q * kRows][c], y, acc[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            const int i = i0 + ty + q * kRows, k = k0 + tx;
+            if (i < m && k <= i) M[(size_t)i * m + k] = acc[q];
+        }
+    }
+}
+
+// M = A O^2 A' for the cached operator.
+template <typename T>
+__device__ __noinline__ void phase_dense_assemble(const IterParams<T>& P) {
+    if (!P.full_rows) phase_dense_scatter(P);
+    else if (blockDim.x == 1024) dense_syrk<1>(P);
+    else if (blockDim.x == 512) dense_syrk<2>(P);
+    else dense_syrk<4>(P);
 }
 
 // dM <- X' (upper triangle, row-major), 32 x 32 tiles through shared memory.
@@ -2523,8 +2604,6 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
     int l = __ldcg(&ctl->l);
     bool refresh = P.refresh != 0 || status0 == ST_SWITCH;
     int status = ST_RUNNING;
-    long long cg_total = 0;
-    long long nA = 0, nAT = 0, nA64 = 0, nAT64 = 0, ncond = 0, nchk = 0, nA32 = 0, nAT32 = 0;
     // FP32 loop of the single-problem launch: column-blocked CG passes, and
     // FP32 outer passes while P.outer32 is on (until ctl->outer32_end is set)
     const bool cbcg = sizeof(T) == 4 && P.Acb.nblocks > 0 && P.ATcb.nblocks > 0;
@@ -2538,8 +2617,15 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         L.eta = __ldcg(&ctl->eta);
         L.best_mx = INFINITY;
         L.flat_checks = 0;
+        L.win_cg = __ldcg(&ctl->win_cg);
+        for (int i = 0; i < CT_COUNT; ++i) L.count[i] = 0;
     }
     __syncthreads();
+    // the pass counters live in shared memory and are kept by thread 0: in
+    // registers they would be spilled around every phase by every thread
+    auto count = [&](int which) {
+        if (threadIdx.x == 0) ++L.count[which];
+    };
     bool ok = true;
     // cached projection operator (FP64 loops only); a factorisation that fails
     // (M singular: rank-deficient A) hands this solve to the CG projection
@@ -2564,9 +2650,7 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
     bool factor_kept = P.own_scratch != 0 && factor_ok;
     bool over = false;                                  // deadline of a time-sliced solve passed
     bool extrap_ok = __ldcg(&ctl->extrap_ok) != 0;
-    long long win_cg = __ldcg(&ctl->win_cg);
     int win_it = __ldcg(&ctl->win_it);
-    long long ndense = 0, nfactor = 0;
     bool abs_fused = false;                             // p, g of the next iteration already formed
     // FP32 outer products on the L2-gather layout (FP32 loop, a segment that
     // ends at a polish level)
@@ -2590,11 +2674,7 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         if (l >= P.max_iter) { status = ACS_MAX_ITER; break; }
         const int lnext = l + 1;
         const bool cond = (lnext == 1) || in_schedule(P, lnext);
-        if (cond) {                                     // a new scaling: a new rental
-            win_cg = 0;
-            win_it = 0;
-        }
-        if (may_switch && !dense && !dense_failed && win_cg > P.switch_budget) {
+        if (may_switch && !dense && !dense_failed && !cond && L.win_cg > P.switch_budget) {
             if (sizeof(T) == 4) {
                 want_dense = true;
                 status = ST_SWITCH;
@@ -2604,6 +2684,8 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
             refresh = true;                                     // factor at this iteration
         }
         if (cond) {                                             // steps 5-14
+            win_it = 0;                                         // a new scaling: a new rental
+            if (threadIdx.x == 0) L.win_cg = 0;
             phase_cond_o(P);
             ACS_SYNC_POST(PH_COND_O, [&](const double* mm) {
                 CondRange R;
@@ -2618,14 +2700,14 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
             });
             phase_cond_apply(P, L.range, true, true);
             ACS_SYNC(PH_COND_APPLY);
-            ++ncond;
+            count(CT_COND);
         } else if (refresh) {
             phase_cond_apply(P, CondRange{0.0, 0.0, 0.0, false}, false, false);
             ACS_SYNC(PH_COND_APPLY);
         }
         if (cond || refresh) {
             phase_btilde(P);
-            ++nA64;
+            count(CT_A64);
             ACS_SYNC_POST(PH_BTILDE, [&](const double* bb) {
                 if (threadIdx.x == 0) L.bad = bb[0] > 0.0;
             });
@@ -2649,12 +2731,12 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                 if (dense) {
                     dense_transpose(sync_smem().dX, sync_smem().dM, P.m);
                     ACS_SYNC(PH_DENSE_INVERSE);
-                    ++nfactor;
+                    count(CT_FACTOR);
                     factor_ok = true;
                 }
             }
             phase_update(P, false, false);                      // q = A_hat' w for the warm start
-            ++nAT64;
+            count(CT_AT64);
             ACS_SYNC(PH_QREFRESH);
             refresh = false;
         }
@@ -2674,18 +2756,18 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         if (dense) {
             // one exact correction: dw = X'(X r0)
             phase_rhs_plain(P);
-            ++nA64;
+            count(CT_A64);
             ACS_SYNC(PH_RHS);
             phase_dense_y(P);
             ACS_SYNC(PH_DENSE_SOLVE);
             phase_dense_x(P);
             ACS_SYNC(PH_DENSE_SOLVE);
-            ++ndense;
+            count(CT_DENSE);
         }
         for (int round = 0; round < (dense ? 0 : P.refine); ++round) {
             if (round > 0) {
                 phase_update(P, false, false);
-                ++nAT64;
+                count(CT_AT64);
                 ACS_SYNC(PH_QREFRESH);
             }
             // the step-relative rule needs a previous step in the same scaling;
@@ -2706,17 +2788,17 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
             };
             if (outer32) {                                      // r0 from an FP32 product
                 phase_rhs_cb(P);
-                ++nA32;
+                count(CT_A32);
                 ACS_SYNC(PH_RHS);
                 phase_rhs_comb(P);
                 ACS_SYNC_POST(PH_RHS_COMB, start_cg);
             } else if (outer32_l2) {
                 phase_rhs_f32(P);                               // r0 from an FP32 product
-                ++nA32;
+                count(CT_A32);
                 ACS_SYNC_POST(PH_RHS, start_cg);
             } else {
                 phase_rhs(P);                                   // r0 in FP64
-                ++nA64;
+                count(CT_A64);
                 ACS_SYNC_POST(PH_RHS, start_cg);
             }
             if (L.bad) { status = ACS_ERR_NUMERICAL; break; }
@@ -2729,16 +2811,16 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                     // the first half, the second half's sums are combined in the
                     // vector step
                     phase_cg_At_cb(P);                          // partial sums of A'u
-                    ++nAT;
+                    count(CT_AT);
                     ACS_SYNC(PH_CG_AT);
                     phase_cg_tcomb(P);                          // t = O^2 A'u, u'Mu
                     ACS_SYNC_POST(PH_CG_TCOMB, step_scalars);
                 } else {
                     phase_cg_At(P);                             // t = O^2 A' u
-                    ++nAT;
+                    count(CT_AT);
                     ACS_SYNC(PH_CG_AT);
                     phase_cg_A(P);                              // au = A t = M u
-                    ++nA;
+                    count(CT_A);
                     ACS_SYNC_POST(PH_CG_A, step_scalars);
                 }
                 if (L.broke) {
@@ -2748,7 +2830,7 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                 }
                 if (cbcg) {
                     phase_cg_A_cb(P);                           // partial sums of A t = M u
-                    ++nA;
+                    count(CT_A);
                     ACS_SYNC(PH_CG_A);
                     phase_cg_vec<T, true>(P);
                 } else {
@@ -2759,8 +2841,10 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
                 if (L.bad) { status = ACS_ERR_NUMERICAL; break; }
             }
             if (!ok || status == ACS_ERR_NUMERICAL) break;
-            cg_total += k;
-            win_cg += k;
+            if (threadIdx.x == 0) {
+                L.count[CT_CG] += k;
+                L.win_cg += k;
+            }
             // an FP32 solve that stalls far above its target cannot refine this M
             if ((broke || k >= P.cg_max) && L.far) trouble = true;
         }
@@ -2811,17 +2895,17 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         };
         if (outer32) {                                          // steps 18-21, FP32 product
             phase_update_cb(P);
-            ++nAT32;
+            count(CT_AT32);
             ACS_SYNC(PH_UPDATE);
             phase_update_comb(P, want_xz, fuse_abs);
             ACS_SYNC_POST(PH_UPD_COMB, after_update);
         } else if (outer32_l2) {
             phase_update_f32(P, want_xz, fuse_abs);             // steps 18-21, FP32 product
-            ++nAT32;
+            count(CT_AT32);
             ACS_SYNC_POST(PH_UPDATE, after_update);
         } else {
             phase_update(P, true, want_xz, fuse_abs);          // steps 18-21
-            ++nAT64;
+            count(CT_AT64);
             ACS_SYNC_POST(PH_UPDATE, after_update);
         }
         abs_fused = fuse_abs;
@@ -2838,9 +2922,9 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
 
         if (check) {
             phase_kkt(P);
-            ++nA64;
-            ++nAT64;
-            ++nchk;
+            count(CT_A64);
+            count(CT_AT64);
+            count(CT_CHECK);
             // FP32 outer passes end once the residuals reach outer32_tol, or
             // once they stop falling (the FP32 products' rounding floor): the
             // rest of the solve runs the FP64 passes from the same iterate
@@ -2885,27 +2969,27 @@ __device__ __noinline__ int solve_loop(const IterParams<T>& P, int status0) {
         ctl->status = err != 0 ? err : status;
         if (status == ST_SWITCH && err == 0) ctl->switched_at = l;
         ctl->l = l;
-        ctl->cg_iters += cg_total;
+        ctl->cg_iters += L.count[CT_CG];
         for (int i = 0; i < 6; ++i) ctl->res[i] = L.res[i];
         ctl->ds = L.ds;
         ctl->snorm = L.snorm;
         ctl->eta = L.eta;
-        ctl->n_cg_A += nA;
-        ctl->n_cg_AT += nAT;
-        ctl->n_64_A += nA64;
-        ctl->n_64_AT += nAT64;
-        ctl->n_cond += ncond;
-        ctl->n_checks += nchk;
-        ctl->n_dense_solve += ndense;
-        ctl->n_dense_factor += nfactor;
-        ctl->n_32_A += nA32;
-        ctl->n_32_AT += nAT32;
+        ctl->n_cg_A += L.count[CT_A];
+        ctl->n_cg_AT += L.count[CT_AT];
+        ctl->n_64_A += L.count[CT_A64];
+        ctl->n_64_AT += L.count[CT_AT64];
+        ctl->n_cond += L.count[CT_COND];
+        ctl->n_checks += L.count[CT_CHECK];
+        ctl->n_dense_solve += L.count[CT_DENSE];
+        ctl->n_dense_factor += L.count[CT_FACTOR];
+        ctl->n_32_A += L.count[CT_A32];
+        ctl->n_32_AT += L.count[CT_AT32];
         ctl->outer32_end = outer32_end;
         ctl->stage = (sizeof(T) == 8 || status == ST_SWITCH) ? 1 : 0;
         ctl->dense_on = (dense || want_dense) ? 1 : 0;
         ctl->factor_ok = factor_ok ? 1 : 0;
         ctl->dense_failed = dense_failed ? 1 : 0;
-        ctl->win_cg = win_cg;
+        ctl->win_cg = L.win_cg;
         ctl->win_it = win_it;
         ctl->extrap_ok = extrap_ok ? 1 : 0;
         ctl->bar_gen = sync_smem().gen;

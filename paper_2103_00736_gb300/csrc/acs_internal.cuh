@@ -215,6 +215,7 @@ struct Problem {
     Control* ctl = nullptr;
     Control* ctl_host = nullptr;         // pinned mirror
     int grid32 = 0, grid64 = 0;
+    int small_ctas = 0;                  // CTAs of the one-cluster launch (0: the whole grid)
     bool warm = false;                   // acs_set_state called
     long long solves = 0;                // acs_solve_async calls
     bool state_clobbered = false;        // a polish overwrote the iteration state
@@ -283,6 +284,10 @@ int support_rows(Problem* P, SellMat& out, bool with_f32);
 // its rounding floor).
 int launch_polish(Problem* P, int rounds, double rel);
 int occupancy_grid(Problem* P);
+// The one-cluster launch of small problems (acs_small.cu): its CTAs for this
+// problem (0: use the whole grid), and the launch.
+int small_cluster(const Problem* P);
+cudaError_t launch_small(const IterParams<double>& Q, int ctas, cudaStream_t stream);
 int cb_smem_limit();
 int pass_bench(Problem* P, int kind, int reps, int smem_bytes, double* us);
 int barrier_probe(Problem* P, int n, double* ns_per_barrier, int absent = -1);

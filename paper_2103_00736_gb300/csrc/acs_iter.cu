@@ -82,8 +82,10 @@ barrier_probe_kernel(Control* ctl, unsigned* flags, double* partials, int n, dou
 // layout the problem lacks do nothing.  The iterate state of the problem is
 // left undefined (the next acs_solve starts afresh unless acs_set_state).
 __global__ void __launch_bounds__(kThreads, 1)
-pass_bench_kernel(const __grid_constant__ IterParams<float> P, const __grid_constant__ IterParams<double> P64, int kind,
-                  int reps, double* out_ns) {
+pass_bench_kernel(const __grid_constant__ IterParams<float> P32, const __grid_constant__ IterParams<double> P64_,
+                  int kind, int reps, double* out_ns) {
+    const IterParams<float>& P = stage_params(P32);
+    const IterParams<double>& P64 = stage_params(P64_);
     team_set(blockIdx.x, gridDim.x, &P.ctl->bar_count64, P.partials);
     sync_init(P.ctl->bar_gen);
     if (P.Acb.nblocks > 0) cb_init();
@@ -140,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1) iter_kernel(const __grid_constant
              P.dense ? P.dX : nullptr);
     sync_init(P.ctl->bar_gen);
     if (P.Acb.nblocks > 0) cb_init();
-    solve_loop<T>(P, status0);
+    solve_loop<T>(stage_params(P), status0);
 }
 
 // LP crossover polish of the current iterate (FP64; see polish_loop).
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, 1) polish_kernel(const __grid_consta
                                                              int fp32) {
     team_set(blockIdx.x, gridDim.x, &P.ctl->bar_count64, P.partials, P.dM, P.dX);
     sync_init(P.ctl->bar_gen);
-    polish_loop(P, P32, Q, out, rounds, rel, fp32 != 0);
+    polish_loop(stage_params(P), stage_params(P32), stage_params<double, 1>(Q), out, rounds, rel, fp32 != 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -437,7 +439,7 @@ int launch_solve(Problem* P, double tol, int max_iter) {
     if (P->set.precision == ACS_PREC_FP64 || P->dense == 1) {
         // the cached operator runs in the FP64 loop (exact corrections)
         IterParams<double> Q = make_params<double>(P, tol, max_iter, P->V64);
-        e = launch_iter<double>(P, Q, P->grid64);
+        e = P->small_ctas > 0 ? launch_small(Q, P->small_ctas, st) : launch_iter<double>(P, Q, P->grid64);
     } else {
         IterParams<float> Q = make_params<float>(P, tol, max_iter, P->V32);
         e = launch_iter<float>(P, Q, P->grid32);

@@ -687,6 +687,7 @@ int acs_server_submit(acs_server* h, const acs_instance* I, double tol, int32_t 
                             R->X.H) != ACS_SOLVED)
                 return ACS_ERR_CSR;
             R->X.stored = (long long)R->X.H.A.col.size();
+            R->X.full = nnz == (long long)I->m * I->n;
             Member& M = R->M;
             M.m = I->m; M.n = I->n; M.n_orth = I->n_orthant; M.n_soc = I->n_soc; M.mat = 0;
             M.dense = host::dense_mode(rs, I->m);

@@ -124,18 +124,18 @@ __device__ __noinline__ bool run_member(const BatchArgs& B, int i, double* scrat
     const bool fresh = B.p64[i].refresh == 0;
     const int stage = fresh ? 0 : __ldcg(&ctl->stage);
     if (B.fp64 || B.p64[i].dense == 1 || stage == 1) {   // the cached operator runs in the FP64 loop
-        const IterParams<double>& P = B.p64[i];
+        const IterParams<double>& P = stage_params(B.p64[i]);
         if (fresh) init_member(P);
         if (!grid_sync(&ctl->err)) return false;
         solve_loop<double>(P, ST_RUNNING);
     } else {
-        const IterParams<float>& P = B.p32[i];
+        const IterParams<float>& P = stage_params(B.p32[i]);
         if (fresh) init_member(P);
         if (!grid_sync(&ctl->err)) return false;
         if (solve_loop<float>(P, ST_RUNNING) == ST_SWITCH) {
             // the loop's state is in ctl (written by rank 0): publish it
             if (!grid_sync(&ctl->err)) return false;
-            solve_loop<double>(B.p64[i], ST_SWITCH);
+            solve_loop<double>(stage_params(B.p64[i]), ST_SWITCH);
         }
     }
     // a barrier that timed out leaves the team out of step: stop it
@@ -267,6 +267,7 @@ struct Matrix {       // one distinct A of the batch
     SellMat A{}, AT{};
     DevSell dA{}, dAT{};
     long long stored = 0;
+    bool full = false;              // every row holds every column
 };
 
 struct Member {
@@ -343,6 +344,7 @@ IterParams<T> member_params(const acs_settings& set, const int* d_cond_list, int
     Q.switch_budget = host::switch_budget(set, M.m, M.nnz);
     Q.extrap = set.extrapolation;
     Q.admm = set.splitting == ACS_SPLIT_ADMM ? 1 : 0;
+    Q.full_rows = X.full ? 1 : 0;
     Q.dM = Q.dX = nullptr;                    // team scratch, set by the kernel
     return Q;
 }
