@@ -8,12 +8,21 @@
 // computation live in one file-scope device array of fixed size that every GPU
 // which loads this library holds until the process exits.
 //
-// Scratch layout (doubles): kMaxN entries for A'y, then kMaxBlocks x 8 block
-// partials.  A'y is accumulated by scattering the rows of A (atomic adds), so
-// its summation order, and hence the last bits of r_d, may differ from call to
-// call.  The accumulator is cleared at the start of every call.  Calls that
-// overlap on the GPU (different streams, or another thread) share the array
-// and race; callers must order them.
+// Scratch layout (doubles): two for the counter of finished blocks, kMaxN entries
+// for A'y, then kMaxBlocks x 8 block partials.  A'y is accumulated by scattering
+// the rows of A (atomic adds), so its summation order, and hence the last bits
+// of r_d, may differ from call to call.  The accumulator is cleared at the start
+// of every call.  Calls that overlap on the GPU (different streams, or another
+// thread) share the array and race; callers must order them.
+//
+// What bounds it, at n = 1e6 and 1e7 nonzeros: each nonzero is 12 bytes of the
+// matrix (18 us of HBM), one random read of x, two FP64 operations (32 us of a
+// pipe that does two multiply-adds per clock per SM) and one atomic add in L2.
+// Eight lanes a row make the matrix reads coalesced and keep short rows from
+// idling a warp.  A small problem is latency only, and runs as one kernel on one
+// thread-block cluster instead of four launches.  Measured: n = 1e6 476 ->
+// 160 us, n = 500 29 -> 20 us a call (before: a thread a row, and one thread
+// adding up the 1024 block partials).
 
 #include <math.h>
 #include <mutex>
@@ -23,59 +32,113 @@
 namespace {
 
 constexpr int kMaxN = 1 << 20;                 // largest n accepted (1,048,576): 8 MiB of A'y
-constexpr int kMaxBlocks = 1024;               // grid size of the two reduction kernels
+constexpr int kMaxBlocks = 1024;               // block partials: half for the rows, half for the columns
 constexpr int kVals = 8;                       // partials per block
-constexpr int kThreadsNA = 256;
+constexpr int kThreadsNA = 1024;
+constexpr int kLanes = 8;                      // lanes a row of A, or a cone, is spread over
+constexpr int kHead = 2;                       // doubles before A'y: the counter of finished blocks
+constexpr int kSmallCtas = 8;                  // the one-cluster kernel (a portable cluster size)
+constexpr int kSmallThreads = 512;
 
-__device__ __align__(256) double g_noalloc_scratch[kMaxN + kMaxBlocks * kVals];
+__device__ __align__(256) double g_noalloc_scratch[kHead + kMaxN + kMaxBlocks * kVals];
 
 std::mutex g_setup_mutex;
 
-__device__ __forceinline__ double warp_sum_na(double x) {
+struct Args {
+    int m, n, n_orth, n_soc;
+    const int *rp, *ci;
+    const double *av, *b, *c, *x, *y, *z;
+    const int* soc_off;
+    double *aty, *prow, *pcol, *out;
+    unsigned* done;
+};
+
+// Block-wide sums of NV <= kVals values; the first NV threads write them to out.
+// Inside a warp a lane gives half of its values away at each of the first steps,
+// so that eight values take nine additions a lane (the FP64 pipe is slow).
+template <int NV>
+__device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* out) {
+    constexpr int NP = NV <= 4 ? 4 : 8;
+    __shared__ double sh[32][NP];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double a[NP];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    for (int k = 0; k < NP; ++k) a[k] = k < NV ? v[k < NV ? k : 0] : 0.0;
+    int o = 16;
+#pragma unroll
+    for (int c = NP; c > 1; c >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < c / 2; ++i) {
+            const double give = up ? a[i] : a[i + c / 2], keep = up ? a[i + c / 2] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    __syncthreads();                                     // sh may still be read from an earlier call
+    if ((lane & (32 / NP - 1)) == 0) sh[warp][lane / (32 / NP)] = a[0];
+    __syncthreads();
+    if (warp == 0) {
+        // lane (k, q): value k, warps q, q + 4, ... (4 or 8 lanes a value)
+        constexpr int Q = 32 / NP;
+        const int k = lane / Q, q = lane % Q;
+        double t = 0.0;
+        for (int w = q; w < nw; w += Q) t += sh[w][k];
+#pragma unroll
+        for (int d = Q / 2; d > 0; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+        if (q == 0 && k < NV) out[k] = t;
+    }
+}
+
+__device__ __forceinline__ double lanes_sum(double x) {
+#pragma unroll
+    for (int o = kLanes / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
 }
 
-// Block-wide sums of NV values; thread 0 writes them to out[0..NV).
-template <int NV>
-__device__ void block_sum_store(double (&v)[NV], double* out) {
-    __shared__ double sh[kThreadsNA / 32][NV];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        const double x = warp_sum_na(v[k]);
-        if (lane == 0) sh[warp][k] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double x = 0.0;
-        for (int w = 0; w < kThreadsNA / 32; ++w) x += sh[w][threadIdx.x];
-        out[threadIdx.x] = x;
-    }
-}
-
-// Rows of A: partials ||Ax - b||^2, b'y, ||b||^2; scatter y_i A_ij into aty[j].
-__global__ void __launch_bounds__(kThreadsNA) rows_kernel(int m, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                          const double* __restrict__ av, const double* __restrict__ b,
-                                                          const double* __restrict__ x, const double* __restrict__ y,
-                                                          double* aty, double* partials) {
-    double v[3] = {0.0, 0.0, 0.0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        const int e = rp[i + 1];
-        const double yi = y[i];
-        double s = 0.0;
-        for (int k = rp[i]; k < e; ++k) {
-            const int j = ci[k];
-            s = fma(av[k], x[j], s);
-            atomicAdd(aty + j, av[k] * yi);
+// Rows of A, kLanes lanes a row: v += {||Ax - b||^2, b'y, ||b||^2}; scatter
+// y_i A_ij into aty[j].  t, nt: this thread and the number of threads.
+__device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (&v)[3]) {
+    const int l = t % kLanes;
+    constexpr int U = 4;
+    // every lane of a warp runs the same number of rounds (its rows past m are empty)
+    for (unsigned i0 = (t & ~31) / kLanes; i0 < (unsigned)P.m; i0 += nt / kLanes) {
+        const unsigned i = i0 + (t & 31) / kLanes;
+        int k = 0, e = 0;
+        double yi = 0.0;
+        if (i < (unsigned)P.m) {
+            k = P.rp[i] + l;
+            e = P.rp[i + 1];
+            yi = P.y[i];
         }
-        const double d = s - b[i];
-        v[0] += d * d;
-        v[1] += b[i] * yi;
-        v[2] += b[i] * b[i];
+        double s = 0.0;
+        for (; k < e; k += U * kLanes) {
+            int j[U];
+            double a[U], xj[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool in = k + u * kLanes < e;
+                j[u] = in ? __ldcs(P.ci + k + u * kLanes) : -1;
+                a[u] = in ? __ldcs(P.av + k + u * kLanes) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) xj[u] = j[u] >= 0 ? P.x[j[u]] : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j[u] >= 0) {
+                    s = fma(a[u], xj[u], s);
+                    atomicAdd(P.aty + j[u], a[u] * yi);
+                }
+        }
+        s = lanes_sum(s);
+        if (l == 0 && i < (unsigned)P.m) {
+            const double bi = P.b[i], d = s - bi;
+            v[0] += d * d;
+            v[1] += bi * yi;
+            v[2] += bi * bi;
+        }
     }
-    block_sum_store<3>(v, partials + blockIdx.x * kVals);
 }
 
 __device__ __forceinline__ double soc_dist2_na(double v1, double t) {
@@ -85,56 +148,119 @@ __device__ __forceinline__ double soc_dist2_na(double v1, double t) {
     return 2.0 * d * d;
 }
 
-// Coordinates and cones: ||A'y + z - c||^2, c'x, ||x||^2, ||z||^2, dist(x,K)^2,
-// dist(z,K)^2, ||c||^2.
-__global__ void __launch_bounds__(kThreadsNA) cols_kernel(int n, int n_orth, int n_soc, const int* __restrict__ soc_off,
-                                                          const double* __restrict__ c, const double* __restrict__ x,
-                                                          const double* __restrict__ z, const double* aty,
-                                                          double* partials) {
-    double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const double d = aty[j] + z[j] - c[j];
+// Coordinates and cones (kLanes lanes a cone): v += {||A'y + z - c||^2, c'x,
+// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}.
+__device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (&v)[7]) {
+    for (int j = t; j < P.n; j += nt) {
+        const double xj = P.x[j], zj = P.z[j], cj = P.c[j];
+        const double d = __ldcg(P.aty + j) + zj - cj;
         v[0] += d * d;
-        v[6] += c[j] * c[j];
-        v[1] += c[j] * x[j];
-        v[2] += x[j] * x[j];
-        v[3] += z[j] * z[j];
-        if (j < n_orth) {
-            if (x[j] < 0.0) v[4] += x[j] * x[j];
-            if (z[j] < 0.0) v[5] += z[j] * z[j];
+        v[6] += cj * cj;
+        v[1] += cj * xj;
+        const double xx = xj * xj, zz = zj * zj;
+        v[2] += xx;
+        v[3] += zz;
+        if (j < P.n_orth) {
+            if (xj < 0.0) v[4] += xx;
+            if (zj < 0.0) v[5] += zz;
         }
     }
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_soc; q += gridDim.x * blockDim.x) {
-        const int a = soc_off[q], e = soc_off[q + 1];
+    const int l = t % kLanes;
+    for (unsigned q0 = (t & ~31) / kLanes; q0 < (unsigned)P.n_soc; q0 += nt / kLanes) {
+        const unsigned q = q0 + (t & 31) / kLanes;
+        int a = 0, e = 0;
+        if (q < (unsigned)P.n_soc) {
+            a = P.soc_off[q];
+            e = P.soc_off[q + 1];
+        }
         double sx = 0.0, sz = 0.0;
-        for (int j = a + 1; j < e; ++j) {
-            sx = fma(x[j], x[j], sx);
-            sz = fma(z[j], z[j], sz);
+        for (int j = a + 1 + l; j < e; j += kLanes) {
+            const double xj = P.x[j], zj = P.z[j];
+            sx = fma(xj, xj, sx);
+            sz = fma(zj, zj, sz);
         }
-        v[4] += soc_dist2_na(x[a], sqrt(sx));
-        v[5] += soc_dist2_na(z[a], sqrt(sz));
+        sx = lanes_sum(sx);
+        sz = lanes_sum(sz);
+        // lane 0 takes x, lane 1 z
+        if (q < (unsigned)P.n_soc && l < 2) {
+            const double d = l == 0 ? soc_dist2_na(P.x[a], sqrt(sx)) : soc_dist2_na(P.z[a], sqrt(sz));
+            if (l == 0) v[4] += d;
+            else v[5] += d;
+        }
     }
-    block_sum_store<7>(v, partials + blockIdx.x * kVals);
 }
 
-// One block: combine the partials in block order, write the six residual values.
-__global__ void finish_kernel(int nb_rows, int nb_cols, const double* prow, const double* pcol, double* out) {
-    if (threadIdx.x != 0) return;
-    double rp = 0, by = 0, bb = 0, rd = 0, cx = 0, xx = 0, zz = 0, dx = 0, dz = 0, cc = 0;
-    for (int k = 0; k < nb_rows; ++k) {
-        rp += prow[k * kVals]; by += prow[k * kVals + 1]; bb += prow[k * kVals + 2];
-    }
-    for (int k = 0; k < nb_cols; ++k) {
-        const double* p = pcol + k * kVals;
-        rd += p[0]; cx += p[1]; xx += p[2]; zz += p[3]; dx += p[4]; dz += p[5]; cc += p[6];
-    }
-    const double bnorm = sqrt(bb), cnorm = sqrt(cc);
-    out[0] = sqrt(rp) / (1.0 + bnorm);
-    out[1] = sqrt(rd) / (1.0 + cnorm);
-    out[2] = fabs(cx - by) / (1.0 + fabs(cx) + fabs(by));
-    out[3] = fmax(sqrt(dx), sqrt(dz)) / (1.0 + fmax(sqrt(xx), sqrt(zz)));
-    out[4] = cx;
-    out[5] = by;
+// One warp: add the blocks' partials (lane l those of blocks l, l + 32, ... in
+// order, then a fixed shuffle tree) and write the six residual values.
+__device__ __forceinline__ void finish_part(int nb_rows, int nb_cols, const double* prow, const double* pcol,
+                                            double* out) {
+    const int lane = threadIdx.x & 31;
+    double s[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) s[k] = 0.0;
+    for (int i = lane; i < nb_rows; i += 32)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] += __ldcg(prow + i * kVals + k);
+    for (int i = lane; i < nb_cols; i += 32)
+#pragma unroll
+        for (int k = 0; k < 7; ++k) s[3 + k] += __ldcg(pcol + i * kVals + k);
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    const double rp = s[0], by = s[1], bb = s[2], rd = s[3], cx = s[4], xx = s[5], zz = s[6], dx = s[7], dz = s[8],
+                 cc = s[9];
+    double r = 0.0;
+    if (lane == 0) r = sqrt(rp) / (1.0 + sqrt(bb));
+    if (lane == 1) r = sqrt(rd) / (1.0 + sqrt(cc));
+    if (lane == 2) r = fabs(cx - by) / (1.0 + fabs(cx) + fabs(by));
+    if (lane == 3) r = fmax(sqrt(dx), sqrt(dz)) / (1.0 + fmax(sqrt(xx), sqrt(zz)));
+    if (lane == 4) r = cx;
+    if (lane == 5) r = by;
+    if (lane < 6) out[lane] = r;
+}
+
+__global__ void __launch_bounds__(kThreadsNA) rows_kernel(const Args P) {
+    double v[3] = {0.0, 0.0, 0.0};
+    rows_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    block_sum_store<3>(v, P.prow + blockIdx.x * kVals);
+}
+
+// The block that ends last combines all partials.
+__global__ void __launch_bounds__(kThreadsNA) cols_kernel(const Args P, int nb_rows) {
+    double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    cols_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    block_sum_store<7>(v, P.pcol + blockIdx.x * kVals);
+    if (threadIdx.x >= 32) return;
+    __threadfence();
+    __syncwarp();
+    unsigned last = 0;
+    if (threadIdx.x == 0) last = atomicAdd(P.done, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    finish_part(nb_rows, (int)gridDim.x, P.prow, P.pcol, P.out);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// A small problem: the whole computation on one cluster.
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads) small_kernel(const Args P) {
+    const int t = blockIdx.x * kSmallThreads + threadIdx.x;
+    constexpr int nt = kSmallCtas * kSmallThreads;
+    for (int j = t; j < P.n; j += nt) P.aty[j] = 0.0;
+    cluster_barrier();
+    double v[3] = {0.0, 0.0, 0.0};
+    rows_part(P, t, nt, v);
+    block_sum_store<3>(v, P.prow + blockIdx.x * kVals);
+    cluster_barrier();
+    double w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    cols_part(P, t, nt, w);
+    block_sum_store<7>(w, P.pcol + blockIdx.x * kVals);
+    cluster_barrier();
+    if (blockIdx.x == 0 && threadIdx.x < 32) finish_part(kSmallCtas, kSmallCtas, P.prow, P.pcol, P.out);
 }
 
 // Device address of the scratch array in the current device's context,
@@ -168,19 +294,30 @@ extern "C" int acs_kkt_residuals_noalloc(int32_t m, int32_t n, const int32_t* ro
     int err = ACS_SOLVED;
     double* scratch = scratch_for_current_device(&err);
     if (!scratch) return err;
-    double* aty = scratch;
-    double* prow = scratch + kMaxN;
+    Args P{m, n, n_orthant, n_soc, row_ptr, col, val, b, c, x, y, z, soc_offsets, scratch + kHead,
+           scratch + kHead + kMaxN, scratch + kHead + kMaxN + (kMaxBlocks / 2) * kVals, residuals,
+           reinterpret_cast<unsigned*>(scratch)};
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // block counts in 64-bit arithmetic (m + kThreadsNA - 1 may exceed INT32_MAX)
-    const long long rows_need = ((long long)m + kThreadsNA - 1) / kThreadsNA;
+    // One cluster while even a full matrix is little work for its eight SMs (the
+    // number of nonzeros is on the device): m n <= 2^19 is at most 2^16
+    // multiply-adds a product on each, 16 us of FP64 pipe for both, against about
+    // 12 us of launches saved; a sparse problem of that size is latency only.
+    if ((long long)m * n <= (1LL << 19)) {
+        small_kernel<<<kSmallCtas, kSmallThreads, 0, st>>>(P);
+        return cudaGetLastError() == cudaSuccess ? ACS_SOLVED : ACS_ERR_CUDA;
+    }
+    // block counts in 64-bit arithmetic; at most two blocks of 1024 threads on
+    // each of 152 SMs, and never more than the scratch has partials for
+    const long long most = 304 < kMaxBlocks / 2 ? 304 : kMaxBlocks / 2;
+    const long long rows_need = ((long long)m * kLanes + kThreadsNA - 1) / kThreadsNA;
     const long long cols_need = ((long long)n + kThreadsNA - 1) / kThreadsNA;
-    const int nb_rows = (int)(rows_need < kMaxBlocks / 2 ? rows_need : kMaxBlocks / 2);
-    const int nb_cols = (int)(cols_need < kMaxBlocks / 2 ? cols_need : kMaxBlocks / 2);
-    double* pcol = prow + (kMaxBlocks / 2) * kVals;
-    if (cudaMemsetAsync(aty, 0, sizeof(double) * (size_t)n, st) != cudaSuccess) return ACS_ERR_CUDA;
-    rows_kernel<<<nb_rows, kThreadsNA, 0, st>>>(m, row_ptr, col, val, b, x, y, aty, prow);
-    cols_kernel<<<nb_cols, kThreadsNA, 0, st>>>(n, n_orthant, n_soc, soc_offsets, c, x, z, aty, pcol);
-    finish_kernel<<<1, 32, 0, st>>>(nb_rows, nb_cols, prow, pcol, residuals);
+    const long long soc_need = ((long long)n_soc * kLanes + kThreadsNA - 1) / kThreadsNA;
+    const long long wide = cols_need > soc_need ? cols_need : soc_need;
+    const int nb_rows = (int)(rows_need < most ? rows_need : most);
+    const int nb_cols = (int)(wide < most ? wide : most);
+    if (cudaMemsetAsync(scratch, 0, sizeof(double) * ((size_t)n + kHead), st) != cudaSuccess) return ACS_ERR_CUDA;
+    rows_kernel<<<nb_rows, kThreadsNA, 0, st>>>(P);
+    cols_kernel<<<nb_cols, kThreadsNA, 0, st>>>(P, nb_rows);
     if (cudaGetLastError() != cudaSuccess) return ACS_ERR_CUDA;
     return ACS_SOLVED;
 }
