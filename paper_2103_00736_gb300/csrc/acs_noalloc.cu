@@ -21,7 +21,7 @@
 // Eight lanes a row make the matrix reads coalesced and keep short rows from
 // idling a warp.  A small problem is latency only, and runs as one kernel on one
 // thread-block cluster instead of four launches.  Measured: n = 1e6 476 ->
-// 160 us, n = 500 29 -> 20 us a call (before: a thread a row, and one thread
+// 160 us, n = 500 28 -> 16 us a call (before: a thread a row, and one thread
 // adding up the 1024 block partials).
 
 #include <math.h>
@@ -53,12 +53,12 @@ struct Args {
     unsigned* done;
 };
 
-// Block-wide sums of NV <= kVals values; the first NV threads write them to out.
+// Block-wide sums of NV <= 16 values; the first NV threads write them to out.
 // Inside a warp a lane gives half of its values away at each of the first steps,
 // so that eight values take nine additions a lane (the FP64 pipe is slow).
 template <int NV>
 __device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* out) {
-    constexpr int NP = NV <= 4 ? 4 : 8;
+    constexpr int NP = NV <= 4 ? 4 : NV <= 8 ? 8 : 16;
     __shared__ double sh[32][NP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     double a[NP];
@@ -80,7 +80,7 @@ __device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* o
     if ((lane & (32 / NP - 1)) == 0) sh[warp][lane / (32 / NP)] = a[0];
     __syncthreads();
     if (warp == 0) {
-        // lane (k, q): value k, warps q, q + 4, ... (4 or 8 lanes a value)
+        // lane (k, q): value k, warps q, q + Q, ... (Q lanes a value)
         constexpr int Q = 32 / NP;
         const int k = lane / Q, q = lane % Q;
         double t = 0.0;
@@ -97,8 +97,9 @@ __device__ __forceinline__ double lanes_sum(double x) {
     return x;
 }
 
-// Rows of A, kLanes lanes a row: v += {||Ax - b||^2, b'y, ||b||^2}; scatter
-// y_i A_ij into aty[j].  t, nt: this thread and the number of threads.
+// Rows of A, kLanes lanes a row: kDot: v += {||Ax - b||^2, b'y, ||b||^2};
+// kScatter: y_i A_ij into aty[j].  t, nt: this thread and the number of threads.
+template <bool kDot, bool kScatter>
 __device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (&v)[3]) {
     const int l = t % kLanes;
     constexpr int U = 4;
@@ -123,14 +124,15 @@ __device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (
                 a[u] = in ? __ldcs(P.av + k + u * kLanes) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) xj[u] = j[u] >= 0 ? P.x[j[u]] : 0.0;
+            for (int u = 0; u < U; ++u) xj[u] = kDot && j[u] >= 0 ? P.x[j[u]] : 0.0;
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (j[u] >= 0) {
-                    s = fma(a[u], xj[u], s);
-                    atomicAdd(P.aty + j[u], a[u] * yi);
+                    if (kDot) s = fma(a[u], xj[u], s);
+                    if (kScatter) atomicAdd(P.aty + j[u], a[u] * yi);
                 }
         }
+        if (!kDot) continue;
         s = lanes_sum(s);
         if (l == 0 && i < (unsigned)P.m) {
             const double bi = P.b[i], d = s - bi;
@@ -149,12 +151,16 @@ __device__ __forceinline__ double soc_dist2_na(double v1, double t) {
 }
 
 // Coordinates and cones (kLanes lanes a cone): v += {||A'y + z - c||^2, c'x,
-// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}.
+// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}; kRest: all but the first.
+template <bool kDual, bool kRest>
 __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (&v)[7]) {
     for (int j = t; j < P.n; j += nt) {
         const double xj = P.x[j], zj = P.z[j], cj = P.c[j];
-        const double d = __ldcg(P.aty + j) + zj - cj;
-        v[0] += d * d;
+        if (kDual) {
+            const double d = __ldcg(P.aty + j) + zj - cj;
+            v[0] += d * d;
+        }
+        if (!kRest) continue;
         v[6] += cj * cj;
         v[1] += cj * xj;
         const double xx = xj * xj, zz = zj * zj;
@@ -165,6 +171,7 @@ __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (
             if (zj < 0.0) v[5] += zz;
         }
     }
+    if (!kRest) return;
     const int l = t % kLanes;
     for (unsigned q0 = (t & ~31) / kLanes; q0 < (unsigned)P.n_soc; q0 += nt / kLanes) {
         const unsigned q = q0 + (t & 31) / kLanes;
@@ -190,6 +197,29 @@ __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (
     }
 }
 
+// One warp: the six residual values from the sums {||Ax - b||^2, b'y, ||b||^2,
+// then those of cols_part}, the same in every lane.
+__device__ __forceinline__ void write_residuals(const double (&s)[10], double* out) {
+    const int lane = threadIdx.x & 31;
+    const double by = s[1], cx = s[4];
+    // lane 0: r_p, 1: r_d, 2: r_gap, 3: r_cone, as one quotient of each lane's own
+    double num = lane == 1 ? s[3] : s[0], den = lane == 1 ? s[9] : s[2];
+    if (lane == 3) {
+        num = fmax(s[7], s[8]);                          // the root is monotone
+        den = fmax(s[5], s[6]);
+    }
+    num = sqrt(num);
+    den = 1.0 + sqrt(den);
+    if (lane == 2) {
+        num = fabs(cx - by);
+        den = 1.0 + fabs(cx) + fabs(by);
+    }
+    double r = num / den;
+    if (lane == 4) r = cx;
+    if (lane == 5) r = by;
+    if (lane < 6) out[lane] = r;
+}
+
 // One warp: add the blocks' partials (lane l those of blocks l, l + 32, ... in
 // order, then a fixed shuffle tree) and write the six residual values.
 __device__ __forceinline__ void finish_part(int nb_rows, int nb_cols, const double* prow, const double* pcol,
@@ -208,28 +238,19 @@ __device__ __forceinline__ void finish_part(int nb_rows, int nb_cols, const doub
     for (int k = 0; k < 10; ++k)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
-    const double rp = s[0], by = s[1], bb = s[2], rd = s[3], cx = s[4], xx = s[5], zz = s[6], dx = s[7], dz = s[8],
-                 cc = s[9];
-    double r = 0.0;
-    if (lane == 0) r = sqrt(rp) / (1.0 + sqrt(bb));
-    if (lane == 1) r = sqrt(rd) / (1.0 + sqrt(cc));
-    if (lane == 2) r = fabs(cx - by) / (1.0 + fabs(cx) + fabs(by));
-    if (lane == 3) r = fmax(sqrt(dx), sqrt(dz)) / (1.0 + fmax(sqrt(xx), sqrt(zz)));
-    if (lane == 4) r = cx;
-    if (lane == 5) r = by;
-    if (lane < 6) out[lane] = r;
+    write_residuals(s, out);
 }
 
 __global__ void __launch_bounds__(kThreadsNA) rows_kernel(const Args P) {
     double v[3] = {0.0, 0.0, 0.0};
-    rows_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    rows_part<true, true>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
     block_sum_store<3>(v, P.prow + blockIdx.x * kVals);
 }
 
 // The block that ends last combines all partials.
 __global__ void __launch_bounds__(kThreadsNA) cols_kernel(const Args P, int nb_rows) {
     double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    cols_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    cols_part<true, true>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
     block_sum_store<7>(v, P.pcol + blockIdx.x * kVals);
     if (threadIdx.x >= 32) return;
     __threadfence();
@@ -246,21 +267,47 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// A small problem: the whole computation on one cluster.
+// A small problem: the whole computation on one cluster, in the fewest steps one
+// after the other: everything that does not need A'y comes first, together with
+// clearing it, then the scatter, then r_d; ten sums a CTA go to CTA 0 through
+// distributed shared memory.
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads) small_kernel(const Args P) {
+    __shared__ double sums[10], all[kSmallCtas][10];
     const int t = blockIdx.x * kSmallThreads + threadIdx.x;
     constexpr int nt = kSmallCtas * kSmallThreads;
     for (int j = t; j < P.n; j += nt) P.aty[j] = 0.0;
+    double v[3] = {0.0, 0.0, 0.0}, w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    rows_part<true, false>(P, t, nt, v);
+    cols_part<false, true>(P, t, nt, w);
     cluster_barrier();
-    double v[3] = {0.0, 0.0, 0.0};
-    rows_part(P, t, nt, v);
-    block_sum_store<3>(v, P.prow + blockIdx.x * kVals);
+    rows_part<false, true>(P, t, nt, v);
     cluster_barrier();
-    double w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    cols_part(P, t, nt, w);
-    block_sum_store<7>(w, P.pcol + blockIdx.x * kVals);
+    cols_part<true, false>(P, t, nt, w);
+    const double both[10] = {v[0], v[1], v[2], w[0], w[1], w[2], w[3], w[4], w[5], w[6]};
+    block_sum_store<10>(both, sums);
+    if (threadIdx.x < 32) {
+        __syncwarp();
+        if (threadIdx.x < 10) {
+            unsigned remote;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                         : "=r"(remote)
+                         : "r"((unsigned)__cvta_generic_to_shared(&all[blockIdx.x][threadIdx.x])));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(sums[threadIdx.x]) : "memory");
+        }
+    }
     cluster_barrier();
-    if (blockIdx.x == 0 && threadIdx.x < 32) finish_part(kSmallCtas, kSmallCtas, P.prow, P.pcol, P.out);
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        double s[10];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) {
+            s[k] = lane < kSmallCtas ? all[lane][k] : 0.0;
+#pragma unroll
+            for (int o = kSmallCtas / 2; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+            s[k] = __shfl_sync(0xffffffffu, s[k], 0);
+        }
+        write_residuals(s, P.out);
+    }
 }
 
 // Device address of the scratch array in the current device's context,
