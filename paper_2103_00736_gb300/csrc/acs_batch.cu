@@ -335,6 +335,7 @@ int prepare_members(Batch* B, int count, const acs_instance* members, int* bad) 
             M.soc_off.resize(I.n_soc + 1);
             M.soc_off[0] = I.n_orthant;
             for (int k = 0; k < I.n_soc; ++k) M.soc_off[k + 1] = M.soc_off[k] + I.soc_dims[k];
+            M.soc_lanes = host::soc_lanes(M.n_soc, M.soc_off.data());
             double bn = 0, cn = 0;
             for (int r = 0; r < I.m; ++r) bn += I.b[r] * I.b[r];
             for (int j = 0; j < I.n; ++j) cn += I.c[j] * I.c[j];

@@ -520,6 +520,7 @@ int acs_problem_create(int32_t m, int32_t n, const int64_t* row_ptr, const int32
     const HostSell& HT = H.AT;
     const std::vector<double>& bperm = H.bperm;
     const std::vector<int>& off = H.soc_off;
+    P->soc_lanes = acs::host::soc_lanes(n_soc, off.data());
 
     if (!on_device && (acs::host::no_throw([&] { return upload_sell(P, HA, P->A, !cb_ok); }) ||
                        acs::host::no_throw([&] { return upload_sell(P, HT, P->AT, !cb_ok); }))) {

@@ -138,7 +138,13 @@ __device__ __forceinline__ int team_rank() { return sync_smem().team_rank; }
 __device__ __forceinline__ int team_size() { return sync_smem().team_size; }
 __device__ __forceinline__ int global_tid() { return team_rank() * (int)blockDim.x + (int)threadIdx.x; }
 __device__ __forceinline__ int global_threads() { return team_size() * (int)blockDim.x; }
-__device__ __forceinline__ int global_warp() { return global_tid() >> 5; }
+// Warps are numbered across the CTAs first, so that work of fewer units than the
+// team has warps (rows of a dense problem, cones), or of a fraction more than
+// a multiple of them, spreads over all SMs instead of filling the first CTAs:
+// with 2320 rows on 152 x 32 warps, 73 SMs did everything.
+__device__ __forceinline__ int global_warp() {
+    return (int)(threadIdx.x >> 5) * team_size() + team_rank();
+}
 __device__ __forceinline__ int global_warps() { return global_threads() >> 5; }
 
 // The parameter block of a solve, copied to shared memory once per launch or
@@ -633,8 +639,47 @@ __device__ __forceinline__ void sell_rows_g(const SellMat& M, const V* __restric
 #define ACS_CG_U 4
 #endif
 
+// Rows that hold every column in order (dense problems): entry k of a row is
+// column k, so the vector is read in order and no column index is loaded (4 of
+// 8 bytes an entry in FP32, and one of two dependent loads).  Every lane takes
+// the same entries in the same order as above, so the sums are the same.  With
+// fewer rows than warps one row's latency is the pass: eight entries a lane in
+// flight.  Measured with the numbering of global_warp(), m = 2320, n = 2900: FP32
+// pass over A 24.2 -> 14.0 us, over A' 16.6 -> 9.6, FP64 residual pass 35.6 ->
+// 22.7 (phase times, barrier included).
+template <typename T, typename V, typename Gather, typename Epi>
+__device__ __forceinline__ void dense_rows(const SellMat& M, const V* __restrict__ val, Gather gather, Epi epi) {
+    constexpr int U = 8;
+    const int lane = threadIdx.x & 31;
+    const int g = M.g, ncols = M.full, gl = lane & (g - 1);
+    const int len = (ncols + g - 1) / g, h = 32 / g, nw = global_warps();
+    for (int sl = global_warp(); sl < M.nslices; sl += nw) {
+        const V* v = val + (size_t)sl * len * 32 + lane;
+        T acc = T(0);
+        for (int k = 0; k < len; k += U) {
+            T a[U], x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int j = (k + u) * g + gl;
+                const bool in = j < ncols;
+                a[u] = in ? val_to<T>(ld_stream(v + 32 * (k + u))) : T(0);
+                x[u] = in ? gather(j) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc = fma(a[u], x[u], acc);
+        }
+        for (int o = g / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        const int row = sl * h + lane / g;
+        if (gl == 0 && row < M.nrows) epi(row, acc);
+    }
+}
+
 template <typename T, typename V, typename Gather, typename Epi>
 __device__ __forceinline__ void sell_rows_v(const SellMat& M, const V* val, Gather gather, Epi epi) {
+    if (M.full > 0) {
+        dense_rows<T>(M, val, gather, epi);
+        return;
+    }
     constexpr int U = (sizeof(T) == 4) ? ACS_CG_U : 4;
     switch (M.g) {
         case 1: sell_rows_g<1, U, T>(M, val, gather, epi); break;
@@ -1107,6 +1152,29 @@ __device__ __forceinline__ void cb_stage_only(const CbMat& M, const Src* __restr
 // ---------------------------------------------------------------------------
 
 
+// Lorentz cones, a group of P.soc_lanes lanes (a power of two) each.  The roots
+// and quotients of a cone cost a warp about 60 FP64 instructions of 16 cycles
+// however many of its lanes need them, so eight cones a warp share them instead
+// of one; wider groups where cones are long (soc_lanes() in acs_host.cuh).
+// body(a, e, l, G, sum): cone [a, e), lane l of G; sum adds over the group.  Empty
+// groups run with a = e = 0.  Measured: abs_K of 20000 cones of 3 to 64
+// (and 100000 orthant coordinates) 56 -> 29 us, the KKT check 168 -> 93.
+template <typename P_, typename Body>
+__device__ __forceinline__ void for_cones(const P_& P, Body body) {
+    const int G = P.soc_lanes, per = 32 / G;
+    const int lane = threadIdx.x & 31, l = lane & (G - 1);
+    auto sum = [G](double x) {
+        for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        return x;
+    };
+    for (int c0 = global_warp() * per; c0 < P.n_soc; c0 += global_warps() * per) {
+        const int c = c0 + lane / G;
+        const bool in = c < P.n_soc;
+        const int a = in ? __ldg(P.soc_off + c) : 0, e = in ? __ldg(P.soc_off + c + 1) : 0;
+        body(c, a, e, l, G, sum);
+    }
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum_t(T x) {
 #pragma unroll
@@ -1146,13 +1214,11 @@ __device__ __noinline__ void phase_cond_o(const IterParams<T>& P) {
             vneg = fmax(vneg, -lo);
         }
     }
-    const int lane = threadIdx.x & 31;
-    for (int cI = global_warp(); cI < P.n_soc; cI += global_warps()) {
-        const int a = __ldg(P.soc_off + cI), e = __ldg(P.soc_off + cI + 1);
+    for_cones(P, [&](int cI, int a, int e, int l, int G, auto sum) {
         double ss = 0.0;
-        for (int j = a + 1 + lane; j < e; j += 32) ss = fma(P.x[j], P.x[j], ss);
-        ss = warp_sum(ss);
-        if (lane == 0) {
+        for (int j = a + 1 + l; j < e; j += G) ss = fma(P.x[j], P.x[j], ss);
+        ss = sum(ss);
+        if (l == 0 && a < e) {
             const double o = fabs(P.x[a] - sqrt(ss)) / fabs(P.z[a]);
             const double lo = log(o);
             P.ocone[P.n_orth + cI] = lo;
@@ -1162,7 +1228,7 @@ __device__ __noinline__ void phase_cond_o(const IterParams<T>& P) {
                 vneg = fmax(vneg, -lo);
             }
         }
-    }
+    });
     const double v[3] = {vmax, vneg, good};
     const int op[3] = {1, 1, 0};
     block_partials<3>(v, op, P.partials);
@@ -1201,12 +1267,11 @@ __device__ __noinline__ void phase_cond_apply(const IterParams<T>& P, const Cond
         const double Oj = recompute_O ? cond_scale(P.ocone[j], R) : P.X.O[j];
         cond_apply_coord(P, j, Oj, recast);
     }
-    const int lane = threadIdx.x & 31;
-    for (int cI = global_warp(); cI < P.n_soc; cI += global_warps()) {
-        const int a = __ldg(P.soc_off + cI), e = __ldg(P.soc_off + cI + 1);
+    for_cones(P, [&](int cI, int a, int e, int l, int G, auto) {
+        if (a >= e) return;
         const double Oc = recompute_O ? cond_scale(P.ocone[P.n_orth + cI], R) : P.X.O[a];
-        for (int j = a + lane; j < e; j += 32) cond_apply_coord(P, j, Oc, recast);
-    }
+        for (int j = a + l; j < e; j += G) cond_apply_coord(P, j, Oc, recast);
+    });
 }
 
 // b_tilde = b + mu A (O c_hat), J^{-1} = 1 / diag(A_hat A_hat') (FP64 pass);
@@ -1276,12 +1341,11 @@ __device__ __noinline__ void phase_abs(const IterParams<T>& P, double theta) {
         X.p[j] = pj;
         X.g[j] = X.O[j] * (pj + extrap_q(X, j, theta, save));
     }
-    const int lane = threadIdx.x & 31;
-    for (int cI = global_warp(); cI < P.n_soc; cI += global_warps()) {
-        const int a = __ldg(P.soc_off + cI), e = __ldg(P.soc_off + cI + 1);
+    for_cones(P, [&](int, int a, int e, int l, int G, auto sum) {
         double ss = 0.0;
-        for (int j = a + 1 + lane; j < e; j += 32) ss = fma(X.s[j], X.s[j], ss);
-        ss = warp_sum(ss);
+        for (int j = a + 1 + l; j < e; j += G) ss = fma(X.s[j], X.s[j], ss);
+        ss = sum(ss);
+        if (a >= e) return;
         const double t = sqrt(ss);
         const double v1 = X.s[a];
         double ftail, head;
@@ -1289,12 +1353,12 @@ __device__ __noinline__ void phase_abs(const IterParams<T>& P, double theta) {
         else if (t <= -v1) { ftail = -1.0; head = -v1; }
         else { ftail = v1 / t; head = t; }
         const double Oc = X.O[a];
-        for (int j = a + lane; j < e; j += 32) {
+        for (int j = a + l; j < e; j += G) {
             const double pj = (j == a) ? head : ftail * X.s[j];
             X.p[j] = pj;
             X.g[j] = Oc * (pj + extrap_q(X, j, theta, save));
         }
-    }
+    });
 }
 
 // FP64 residual of the projection system r0 = b_tilde - A g (g = O(p + q),
@@ -1587,12 +1651,11 @@ template <typename T>
 __device__ __noinline__ void phase_admm_soc(const IterParams<T>& P, bool want_xz) {
     double ds2 = 0.0, ss2 = 0.0;
     const Outer& X = P.X;
-    const int lane = threadIdx.x & 31;
-    for (int cI = global_warp(); cI < P.n_soc; cI += global_warps()) {
-        const int a0 = __ldg(P.soc_off + cI), e = __ldg(P.soc_off + cI + 1);
+    for_cones(P, [&](int, int a0, int e, int l, int G, auto sum) {
         double tt = 0.0;
-        for (int j = a0 + 1 + lane; j < e; j += 32) tt = fma(X.p[j], X.p[j], tt);
-        tt = warp_sum(tt);
+        for (int j = a0 + 1 + l; j < e; j += G) tt = fma(X.p[j], X.p[j], tt);
+        tt = sum(tt);
+        if (a0 >= e) return;
         const double t = sqrt(tt);
         const double v1 = X.p[a0];
         double ftail, head;
@@ -1600,7 +1663,7 @@ __device__ __noinline__ void phase_admm_soc(const IterParams<T>& P, bool want_xz
         else if (t <= -v1) { ftail = -1.0; head = -v1; }
         else { ftail = v1 / t; head = t; }
         const double Oc = X.O[a0];
-        for (int j = a0 + lane; j < e; j += 32) {
+        for (int j = a0 + l; j < e; j += G) {
             const double a = X.p[j];
             const double aa = (j == a0) ? head : ftail * a;
             const double so = X.s[j];
@@ -1613,7 +1676,7 @@ __device__ __noinline__ void phase_admm_soc(const IterParams<T>& P, bool want_xz
                 P.z[j] = (aa - a) / (2.0 * P.mu * Oc);
             }
         }
-    }
+    });
     const double v[2] = {ds2, ss2};
     const int op[2] = {0, 0};
     block_partials<2>(v, op, P.partials);
@@ -1661,27 +1724,30 @@ __device__ __noinline__ void phase_kkt(const IterParams<T>& P) {
         if (xj < 0.0) dx += xj * xj;
         if (zj < 0.0) dz += zj * zj;
     }
-    const int lane = threadIdx.x & 31;
-    for (int cI = global_warp(); cI < P.n_soc; cI += global_warps()) {
-        const int a = __ldg(P.soc_off + cI), e = __ldg(P.soc_off + cI + 1);
-        double sx = 0.0, sz = 0.0, scx = 0.0;
-        for (int j = a + 1 + lane; j < e; j += 32) {
-            sx = fma(x[j], x[j], sx);
-            sz = fma(z[j], z[j], sz);
-            scx = fma(P.c[j], x[j], scx);
+    for_cones(P, [&](int, int a, int e, int l, int G, auto sum) {
+        double sx = 0.0, sz = 0.0;
+        for (int j = a + l; j < e; j += G) {
+            const double xj = x[j], zj = z[j];
+            cx = fma(P.c[j], xj, cx);
+            if (j > a) {
+                sx = fma(xj, xj, sx);
+                sz = fma(zj, zj, sz);
+            }
         }
-        sx = warp_sum(sx);
-        sz = warp_sum(sz);
-        scx = warp_sum(scx);
-        if (lane == 0) {
-            const double xa = x[a], za = z[a];
-            cx += scx + P.c[a] * xa;
-            xx += sx + xa * xa;
-            zz += sz + za * za;
-            dx += soc_dist2(xa, sqrt(sx));
-            dz += soc_dist2(za, sqrt(sz));
+        sx = sum(sx);
+        sz = sum(sz);
+        if (l < 2 && a < e) {                            // lane 0 takes x, lane 1 z
+            const double s2 = l == 0 ? sx : sz, v1 = l == 0 ? x[a] : z[a];
+            const double d2 = soc_dist2(v1, sqrt(s2)), n2 = s2 + v1 * v1;
+            if (l == 0) {
+                xx += n2;
+                dx += d2;
+            } else {
+                zz += n2;
+                dz += d2;
+            }
         }
-    }
+    });
     const double v[8] = {rp, rd, cx, by, dx, dz, xx, zz};
     const int op[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     block_partials<8>(v, op, P.partials);

@@ -151,6 +151,20 @@ inline int validate(int32_t m, int32_t n, const int64_t* row_ptr, const int32_t*
     return ACS_SOLVED;
 }
 
+// Lanes that share one Lorentz cone: enough that the longest cone takes no more
+// than 64 rounds (a lone long cone must not serialise a few lanes), and no fewer
+// than 4 (a 32-byte sector of FP64 values), else eight entries a lane of the
+// mean cone.
+inline int soc_lanes(int n_soc, const int* off) {
+    if (n_soc <= 0) return 32;
+    int longest = 0;
+    for (int i = 0; i < n_soc; ++i) longest = std::max(longest, off[i + 1] - off[i]);
+    const double mean = (double)(off[n_soc] - off[0]) / n_soc;
+    int g = 4;
+    while (g < 32 && (longest > 64 * g || mean > 12.0 * g)) g *= 2;
+    return g;
+}
+
 constexpr int kDenseLimit = 4096;   // largest m for the cached dense projection operator
 constexpr int kDenseRowsLimit = 16384;   // ... when every row of A is full (tiled assembly of M)
 

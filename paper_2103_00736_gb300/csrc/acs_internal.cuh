@@ -98,6 +98,7 @@ struct Inner {
 // contiguous.  Rows shorter than G*slen[sl] are padded with (col 0, val 0).
 struct SellMat {
     int nrows, nslices, g;
+    int full;              // > 0: every row holds all of this many columns, in order
     const int* sptr;       // [nslices + 1] start of each slice
     const int* slen;       // [nslices] 32-entry chunks in the slice
     const int* col;        // [sptr[nslices]]
@@ -134,6 +135,7 @@ struct IterParams {
     int m, n, n_orth, n_soc;
     SellMat A, AT;                                    // A (rows relabelled) and A'
     const int* soc_off;                               // n_soc + 1 absolute offsets
+    int soc_lanes;                                    // lanes that share one Lorentz cone
     const double* b; const double* c;
     double bnorm, cnorm;
     Outer X;
@@ -187,6 +189,7 @@ void dev_release(int device, void* p, size_t bytes);
 
 struct Problem {
     int m = 0, n = 0, nnz = 0, n_orth = 0, n_soc = 0;
+    int soc_lanes = 32;                  // lanes that share one Lorentz cone (host::soc_lanes)
     int device = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;

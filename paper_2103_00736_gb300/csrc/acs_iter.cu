@@ -224,7 +224,10 @@ static IterParams<T> make_params(Problem* P, double tol, int max_iter, const Inn
     IterParams<T> Q{};
     Q.m = P->m; Q.n = P->n; Q.n_orth = P->n_orth; Q.n_soc = P->n_soc;
     Q.A = P->A; Q.AT = P->AT;
+    Q.A.full = P->full_rows ? P->n : 0;
+    Q.AT.full = P->full_rows ? P->m : 0;
     Q.soc_off = P->soc_off;
+    Q.soc_lanes = P->soc_lanes;
     Q.b = P->b; Q.c = P->c; Q.bnorm = P->bnorm; Q.cnorm = P->cnorm;
     Q.X = P->X;
     Q.V = V;
@@ -400,7 +403,7 @@ int launch_polish(Problem* P, int rounds, double rel) {
         // CG corrections: the passes over the rows of A run on A_B, the rows of
         // A restricted to the support's columns (the other columns carry
         // O_j = 0); those over A' skip the rows off the support
-        SellMat AB;
+        SellMat AB{};
         const int rc = support_rows(P, AB, fp32 != 0);
         if (rc != ACS_SOLVED) return rc;
         Q.A = AB;

@@ -695,6 +695,7 @@ int acs_server_submit(acs_server* h, const acs_instance* I, double tol, int32_t 
             M.b = R->X.H.bperm;
             M.c.assign(I->c, I->c + I->n);
             M.soc_off = R->X.H.soc_off;
+            M.soc_lanes = host::soc_lanes(M.n_soc, M.soc_off.data());
             M.bnorm = R->X.H.bnorm;
             M.cnorm = R->X.H.cnorm;
             Pool dry;

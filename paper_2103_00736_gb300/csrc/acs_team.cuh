@@ -276,6 +276,7 @@ struct Member {
     long long nnz = 0;
     std::vector<double> b, c;
     std::vector<int> soc_off;
+    int soc_lanes = 32;
     double bnorm = 0, cnorm = 0;
     // device pointers inside the pool
     double *db = nullptr, *dc = nullptr, *x = nullptr, *z = nullptr, *ocone = nullptr;
@@ -320,7 +321,10 @@ IterParams<T> member_params(const acs_settings& set, const int* d_cond_list, int
     IterParams<T> Q{};
     Q.m = M.m; Q.n = M.n; Q.n_orth = M.n_orth; Q.n_soc = M.n_soc;
     Q.A = X.A; Q.AT = X.AT;
+    Q.A.full = X.full ? M.n : 0;
+    Q.AT.full = X.full ? M.m : 0;
     Q.soc_off = M.dsoc;
+    Q.soc_lanes = M.soc_lanes;
     Q.b = M.db; Q.c = M.dc; Q.bnorm = M.bnorm; Q.cnorm = M.cnorm;
     Q.X = M.X;
     Q.V = V;
