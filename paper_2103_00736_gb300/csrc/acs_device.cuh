@@ -644,7 +644,7 @@ __device__ __forceinline__ void sell_rows_g(const SellMat& M, const V* __restric
 // 8 bytes an entry in FP32, and one of two dependent loads).  Every lane takes
 // the same entries in the same order as above, so the sums are the same.  With
 // fewer rows than warps one row's latency is the pass: eight entries a lane in
-// flight.  Measured with the numbering of global_warp(), m = 2320, n = 2900: FP32
+// flight (sixteen in FP32 gave nothing more).  Measured with the numbering of global_warp(), m = 2320, n = 2900: FP32
 // pass over A 24.2 -> 14.0 us, over A' 16.6 -> 9.6, FP64 residual pass 35.6 ->
 // 22.7 (phase times, barrier included).
 template <typename T, typename V, typename Gather, typename Epi>
@@ -1547,12 +1547,12 @@ __device__ __noinline__ void phase_cg_vec(const IterParams<T>& P) {
 // q just formed -- the values phase_abs would compute there.
 template <typename T>
 __device__ __forceinline__ void update_epi(const IterParams<T>& P, int j, double sum, bool update, bool want_xz,
-                                           double& ds2, double& ss2, bool fuse_abs = false) {
+                                           double& ds2, double& ss2, bool fuse_abs, bool admm) {
     const double Oj = P.X.O[j];
     const double qj = Oj * sum;
     P.X.q[j] = qj;
     if (!update) P.X.g[j] = Oj * (P.X.p[j] + qj);   // right-hand side input of a refinement round
-    if (update && P.admm) {
+    if (update && admm) {
         // ADMM form (Section III-B), as Douglas-Rachford splitting with the two
         // proximal steps in the other order: p = s = zeta, q = A_hat' w with
         // w = M^{-1}(b_tilde - A_hat zeta), so zeta - mu c_hat + q is the
@@ -1607,14 +1607,35 @@ __device__ __forceinline__ void update_partials(double ds2, double ss2, bool upd
     block_partials<3>(v, op, partials);
 }
 
+// q = A_hat' w and g = O (p + q) alone: the start of a solve in a new scaling, and
+// of a refinement round.  Nothing to reduce.
 template <typename T>
-__device__ __noinline__ void phase_update(const IterParams<T>& P, bool update, bool want_xz, bool fuse_abs = false) {
+__device__ __noinline__ void phase_qrefresh(const IterParams<T>& P) {
+    const double* w = P.X.w;
+    sell_rows<double>(P.AT, [w](int i) { return w[i]; }, [&](int j, double sum) {
+        const double Oj = P.X.O[j];
+        const double qj = Oj * sum;
+        P.X.q[j] = qj;
+        P.X.g[j] = Oj * (P.X.p[j] + qj);
+    });
+}
+
+// The update; the ADMM form is a function of its own, so that the usual one keeps
+// its operands in registers.
+template <typename T, bool kAdmm>
+__device__ __noinline__ void phase_update_form(const IterParams<T>& P, bool want_xz, bool fuse_abs) {
     double ds2 = 0.0, ss2 = 0.0;
     const double* w = P.X.w;
     auto gather = [w](int i) { return w[i]; };
-    auto epi = [&](int j, double sum) { update_epi(P, j, sum, update, want_xz, ds2, ss2, fuse_abs); };
+    auto epi = [&](int j, double sum) { update_epi(P, j, sum, true, want_xz, ds2, ss2, fuse_abs, kAdmm); };
     sell_rows<double>(P.AT, gather, epi);
-    update_partials(ds2, ss2, update, P.partials);
+    update_partials(ds2, ss2, true, P.partials);
+}
+template <typename T>
+__device__ __forceinline__ void phase_update(const IterParams<T>& P, bool update, bool want_xz, bool fuse_abs = false) {
+    if (!update) phase_qrefresh(P);
+    else if (P.admm) phase_update_form<T, true>(P, want_xz, fuse_abs);
+    else phase_update_form<T, false>(P, want_xz, fuse_abs);
 }
 
 // The update from an FP32 product A'w on the L2-gather layout (see phase_rhs_f32).
@@ -1623,7 +1644,7 @@ __device__ __noinline__ void phase_update_f32(const IterParams<T>& P, bool want_
     double ds2 = 0.0, ss2 = 0.0;
     const double* w = P.X.w;
     auto gather = [w](int i) { return (float)w[i]; };
-    auto epi = [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs); };
+    auto epi = [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs, P.admm != 0); };
     sell_rows<float>(P.AT, gather, epi);
     update_partials(ds2, ss2, true, P.partials);
 }
@@ -1639,7 +1660,7 @@ template <typename T>
 __device__ __noinline__ void phase_update_comb(const IterParams<T>& P, bool want_xz, bool fuse_abs = false) {
     double ds2 = 0.0, ss2 = 0.0;
     cb_combine(P.ATcb, &P.ctl->err,
-               [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs); });
+               [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs, P.admm != 0); });
     update_partials(ds2, ss2, true, P.partials);
 }
 
@@ -1841,8 +1862,8 @@ constexpr int kCholB = 16;
 constexpr int kTile = 32;
 
 struct DenseShared {
-    double A[kTile][kCholB + 1];       // L_ip rows of a unit (B: then the unit's block)
-    double B[kTile][kCholB + 1];       // L_jp rows (tiles of M), or
+    double A[2][kTile][kCholB + 1];    // L_ip rows of a unit (B: then the unit's block)
+    double B[2][kTile][kCholB + 1];    // L_jp rows (tiles of M), or
                                        // X_p columns, B[j][t] = X[k0 + t][j0 + j]
     double Lq[kCholB][kCholB + 1];     // L[k1.., k0..]
     double D[kCholB][kCholB + 1];      // diagonal block, then its factor
@@ -1910,10 +1931,12 @@ struct DenseUnit {
 };
 
 // The units of the step at k1, numbered from 0: nB1 of kind 0, nB2 of kind 1,
-// then the tiles of X (nt rows of nX) and of M (lower triangle of nt).
+// then the tiles of X (nt rows of nX) and of M (lower triangle of nt).  Numbers
+// fit 32 bits (m <= 16384: 4e5 units); every thread finds its unit, and 64-bit
+// quotients would cost a quarter of a tile's time.
 struct DensePlan {
     int k0, k1, k2, nB1, nB2, nX;
-    long long total;
+    unsigned total;
 };
 __device__ __forceinline__ DensePlan dense_plan(int m, int k1) {
     DensePlan P;
@@ -1924,39 +1947,45 @@ __device__ __forceinline__ DensePlan dense_plan(int m, int k1) {
     P.nB1 = nt;
     P.nX = k1 > 0 ? (k1 + kTile - 1) / kTile : 0;
     P.nB2 = P.nX;
-    P.total = (long long)P.nB1 + P.nB2 + (k1 > 0 ? (long long)nt * P.nX + (long long)nt * (nt + 1) / 2 : 0);
+    P.total = P.nB1 + P.nB2 + (k1 > 0 ? nt * P.nX + nt * (nt + 1) / 2 : 0);
     return P;
 }
-__device__ __forceinline__ DenseUnit dense_unit(const DensePlan& P, long long u) {
+// Row of entry u of a lower triangle stored by rows.
+__device__ __forceinline__ int tri_row(unsigned u) {
+    int r = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
+    while ((unsigned)(r + 1) * (unsigned)(r + 2) / 2u <= u) ++r;
+    while ((unsigned)r * (unsigned)(r + 1) / 2u > u) --r;
+    return r;
+}
+__device__ __forceinline__ DenseUnit dense_unit(const DensePlan& P, unsigned u) {
     DenseUnit U;
-    if (u < P.nB1) {
+    if (u < (unsigned)P.nB1) {
         U.kind = 0;
         U.i0 = P.k2 + (int)u * kTile;
         U.j0 = P.k1;
         return U;
     }
     u -= P.nB1;
-    if (u < P.nB2) {
+    if (u < (unsigned)P.nB2) {
         U.kind = 1;
         U.i0 = P.k1;
         U.j0 = (int)u * kTile;
         return U;
     }
     u -= P.nB2;
-    const long long tx = (long long)P.nB1 * P.nX;
+    const unsigned tx = (unsigned)P.nB1 * (unsigned)P.nX;
     if (u < tx) {
+        const unsigned q = u / (unsigned)P.nX;
         U.kind = 3;
-        U.i0 = P.k2 + (int)(u / P.nX) * kTile;
-        U.j0 = (int)(u % P.nX) * kTile;
+        U.i0 = P.k2 + (int)q * kTile;
+        U.j0 = (int)(u - q * P.nX) * kTile;
         return U;
     }
     u -= tx;
-    int bi = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
-    while ((long long)(bi + 1) * (bi + 2) / 2 <= u) ++bi;
-    while ((long long)bi * (bi + 1) / 2 > u) --bi;
+    const int bi = tri_row(u);
     U.kind = 2;
     U.i0 = P.k2 + bi * kTile;
-    U.j0 = P.k2 + (int)(u - (long long)bi * (bi + 1) / 2) * kTile;
+    U.j0 = P.k2 + (int)(u - (unsigned)bi * (unsigned)(bi + 1) / 2u) * kTile;
     return U;
 }
 
@@ -2002,47 +2031,55 @@ __device__ __forceinline__ void dense_load(const double* M, const double* X, int
     }
 }
 
+// Operands of a unit into buffer `buf`.
 template <int R>
-__device__ __forceinline__ void dense_compute(double* M, double* X, int m, const DensePlan& P, const DenseUnit& U,
-                                              const DenseRegs<R>& G) {
+__device__ __forceinline__ void dense_store(const DenseUnit& U, const DenseRegs<R>& G, int buf) {
     DenseShared& S = dense_smem();
     constexpr int kRows = kTile / R;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        const int r = ty + q * kRows, t = tx & (kCholB - 1);
+        if (tx < kCholB) S.A[buf][r][t] = G.a[q];
+        else if (U.kind == 2) S.B[buf][r][t] = G.a[q];
+        if ((U.kind == 1 || U.kind == 3) && r < kCholB) S.B[buf][tx][r] = G.b[q];
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void dense_compute(double* M, double* X, int m, const DensePlan& P, const DenseUnit& U,
+                                              const double (&c)[R], int buf) {
+    DenseShared& S = dense_smem();
+    constexpr int kRows = kTile / R;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    double(*SA)[kCholB + 1] = S.A[buf];
+    double(*SB)[kCholB + 1] = S.B[buf];
     double acc[R];
 #pragma unroll
-    for (int q = 0; q < R; ++q) acc[q] = G.c[q];
+    for (int q = 0; q < R; ++q) acc[q] = c[q];
     if (P.k0 >= 0) {
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            const int r = ty + q * kRows, t = tx & (kCholB - 1);
-            if (tx < kCholB) S.A[r][t] = G.a[q];
-            else if (U.kind == 2) S.B[r][t] = G.a[q];
-            if ((U.kind == 1 || U.kind == 3) && r < kCholB) S.B[tx][r] = G.b[q];
-        }
-        __syncthreads();
         if (U.kind == 0) {                               // columns of the block: rows of L_q
             if (tx < kCholB)
 #pragma unroll
                 for (int t = 0; t < kCholB; ++t) {
                     const double y = S.Lq[tx][t];
 #pragma unroll
-                    for (int q = 0; q < R; ++q) acc[q] = fma(-S.A[ty + q * kRows][t], y, acc[q]);
+                    for (int q = 0; q < R; ++q) acc[q] = fma(-SA[ty + q * kRows][t], y, acc[q]);
                 }
         } else if (U.kind == 1) {
 #pragma unroll
             for (int q = 0; q < R; ++q)
                 if (ty + q * kRows < kCholB)
 #pragma unroll
-                    for (int t = 0; t < kCholB; ++t) acc[q] = fma(-S.Lq[ty + q * kRows][t], S.B[tx][t], acc[q]);
+                    for (int t = 0; t < kCholB; ++t) acc[q] = fma(-S.Lq[ty + q * kRows][t], SB[tx][t], acc[q]);
         } else {
 #pragma unroll
             for (int t = 0; t < kCholB; ++t) {
-                const double y = S.B[tx][t];
+                const double y = SB[tx][t];
 #pragma unroll
-                for (int q = 0; q < R; ++q) acc[q] = fma(-S.A[ty + q * kRows][t], y, acc[q]);
+                for (int q = 0; q < R; ++q) acc[q] = fma(-SA[ty + q * kRows][t], y, acc[q]);
             }
         }
-        __syncthreads();
     }
     if (U.kind >= 2) {
 #pragma unroll
@@ -2054,10 +2091,11 @@ __device__ __forceinline__ void dense_compute(double* M, double* X, int m, const
         return;
     }
     // kinds 0 and 1: the block through shared memory, times the inverse factor
+    __syncthreads();                                     // the operands are used up
     if (U.kind == 0) {
 #pragma unroll
         for (int q = 0; q < R; ++q)
-            if (tx < kCholB) S.A[ty + q * kRows][tx] = acc[q];
+            if (tx < kCholB) SA[ty + q * kRows][tx] = acc[q];
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[q] = 0.0;
@@ -2066,7 +2104,7 @@ __device__ __forceinline__ void dense_compute(double* M, double* X, int m, const
             for (int t = 0; t < kCholB; ++t) {
                 const double y = S.Di[tx][t];
 #pragma unroll
-                for (int q = 0; q < R; ++q) acc[q] = fma(S.A[ty + q * kRows][t], y, acc[q]);
+                for (int q = 0; q < R; ++q) acc[q] = fma(SA[ty + q * kRows][t], y, acc[q]);
             }
 #pragma unroll
         for (int q = 0; q < R; ++q) {
@@ -2076,7 +2114,7 @@ __device__ __forceinline__ void dense_compute(double* M, double* X, int m, const
     } else {
 #pragma unroll
         for (int q = 0; q < R; ++q)
-            if (ty + q * kRows < kCholB) S.B[tx][ty + q * kRows] = acc[q];
+            if (ty + q * kRows < kCholB) SB[tx][ty + q * kRows] = acc[q];
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < R; ++q) {
@@ -2084,37 +2122,41 @@ __device__ __forceinline__ void dense_compute(double* M, double* X, int m, const
             if (r < kCholB) {
                 double x = 0.0;
 #pragma unroll
-                for (int t = 0; t < kCholB; ++t) x = fma(S.Di[r][t], S.B[tx][t], x);
+                for (int t = 0; t < kCholB; ++t) x = fma(S.Di[r][t], SB[tx][t], x);
                 const int i = U.i0 + r, j = U.j0 + tx;
                 if (i < m && j < P.k1) X[(size_t)i * m + j] = x;
             }
         }
     }
-    __syncthreads();                                     // the operands of the next unit may be stored
 }
 
+// One barrier a unit: its operands go to one of two buffers, and a thread that
+// stores those of the next unit knows from the barrier in between that no one
+// still reads the unit before.
 template <int R>
 __device__ __noinline__ void dense_units(double* M, double* X, int m, int k1) {
     const DensePlan P = dense_plan(m, k1);
-    const int size = team_size();
-    long long u = team_rank();
+    const unsigned size = team_size();
+    unsigned u = team_rank();
     if (u >= P.total) return;                            // CTA-uniform
     DenseUnit U = dense_unit(P, u);
     DenseRegs<R> G;
     dense_load<R>(M, X, m, P, U, G);
-    while (true) {
-        const long long un = u + size;
-        DenseUnit V = U;
-        DenseRegs<R> H = G;
-        if (un < P.total) {
-            V = dense_unit(P, un);
-            dense_load<R>(M, X, m, P, V, H);
+    for (int buf = 0;; buf ^= 1) {
+        dense_store<R>(U, G, buf);
+        double c[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) c[q] = G.c[q];
+        __syncthreads();
+        const DenseUnit V = U;
+        u += size;
+        const bool more = u < P.total;
+        if (more) {
+            U = dense_unit(P, u);
+            dense_load<R>(M, X, m, P, U, G);
         }
-        dense_compute<R>(M, X, m, P, U, G);
-        if (un >= P.total) break;
-        u = un;
-        U = V;
-        G = H;
+        dense_compute<R>(M, X, m, P, V, c, buf);
+        if (!more) break;
     }
 }
 
@@ -2182,16 +2224,15 @@ __device__ __forceinline__ void dense_syrk(const IterParams<T>& P) {
     constexpr int kRows = kTile / R;
     const int m = P.m, n = P.n;
     const int nt = (m + kTile - 1) / kTile;
-    const long long ntile = (long long)nt * (nt + 1) / 2;
+    const unsigned ntile = (unsigned)nt * (unsigned)(nt + 1) / 2u;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int t = tx & (kCholB - 1);
+    int buf = 0;
     const SellMat& A = P.A;
     const int g = A.g, h = 32 / g;
-    for (long long u = team_rank(); u < ntile; u += team_size()) {
-        int bi = (int)((sqrtf(8.0f * (float)u + 1.0f) - 1.0f) * 0.5f);
-        while ((long long)(bi + 1) * (bi + 2) / 2 <= u) ++bi;
-        while ((long long)bi * (bi + 1) / 2 > u) --bi;
-        const int i0 = bi * kTile, k0 = (int)(u - (long long)bi * (bi + 1) / 2) * kTile;
+    for (unsigned u = team_rank(); u < ntile; u += team_size()) {
+        const int bi = tri_row(u);
+        const int i0 = bi * kTile, k0 = (int)(u - (unsigned)bi * (unsigned)(bi + 1) / 2u) * kTile;
         // the lower half of the lanes loads the rows of block i0, the upper half
         // those of k0; entry j of a full row: slice row / h, chunk j / g
         const double* row[R];
@@ -2210,17 +2251,16 @@ __device__ __forceinline__ void dense_syrk(const IterParams<T>& P) {
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[q] = 0.0;
         load(t);
-        for (int j0 = 0; j0 < n; j0 += kCholB) {
-            __syncthreads();                             // the previous slab is used up
+        for (int j0 = 0; j0 < n; j0 += kCholB, buf ^= 1) {
 #pragma unroll
-            for (int q = 0; q < R; ++q) (tx < kCholB ? S.A : S.B)[ty + q * kRows][t] = v[q];
+            for (int q = 0; q < R; ++q) (tx < kCholB ? S.A[buf] : S.B[buf])[ty + q * kRows][t] = v[q];
             __syncthreads();
             if (j0 + kCholB < n) load(j0 + kCholB + t);
 #pragma unroll
             for (int c = 0; c < kCholB; ++c) {
-                const double y = S.B[tx][c];
+                const double y = S.B[buf][tx][c];
 #pragma unroll
-                for (int q = 0; q < R; ++q) acc[q] = fma(S.A[ty + q * kRows][c], y, acc[q]);
+                for (int q = 0; q < R; ++q) acc[q] = fma(S.A[buf][ty + q * kRows][c], y, acc[q]);
             }
         }
 #pragma unroll
@@ -2246,9 +2286,9 @@ static __device__ __noinline__ void dense_transpose(const double* X, double* Mt,
     double(*tile)[kTile + 1] = reinterpret_cast<double(*)[kTile + 1]>(&S);   // 8.4 KB of its 13
     const int nt = (m + kTile - 1) / kTile;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (long long u = team_rank(); u < (long long)nt * nt; u += team_size()) {
-        const int i0 = (int)(u / nt) * kTile, j0 = (int)(u % nt) * kTile;
-        if (j0 > i0) continue;                           // CTA-uniform
+    for (unsigned u = team_rank(); u < (unsigned)nt * (unsigned)(nt + 1) / 2u; u += team_size()) {
+        const int bi = tri_row(u);
+        const int i0 = bi * kTile, j0 = (int)(u - (unsigned)bi * (unsigned)(bi + 1) / 2u) * kTile;
         __syncthreads();
         for (int r = ty; r < kTile; r += nw)
             tile[r][tx] = (i0 + r < m && j0 + tx <= i0 + r) ? __ldcg(X + (size_t)(i0 + r) * m + j0 + tx) : 0.0;
