@@ -66,6 +66,8 @@ struct Batch {
     bool graph_ok = false, last_graph = false;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     std::vector<Control> ctl_host;
+    char* stage = nullptr;            // pinned: a member's control block and results on their way out
+    size_t stage_bytes = 0;           //   (bytes of the results' part)
 };
 
 namespace {
@@ -223,13 +225,14 @@ void layout(Batch* B, Pool& P) {
     // state region
     for (Member& M : B->mem) {
         const int m = M.m, n = M.n;
-        M.x = P.take<double>(n);
+        M.x = P.take<double>(n);                         // x, z, w: read back in one copy
         M.z = P.take<double>(n);
+        M.X.w = P.take<double>(m);
         M.ocone = P.take<double>((size_t)M.n_orth + M.n_soc);
         Outer& X = M.X;
         X.s = P.take<double>(n); X.p = P.take<double>(n); X.g = P.take<double>(n);
         X.q = P.take<double>(n); X.chat = P.take<double>(n); X.O = P.take<double>(n);
-        X.w = P.take<double>(m); X.btil = P.take<double>(m);
+        X.btil = P.take<double>(m);
         X.wp = P.take<double>(m); X.qp = P.take<double>(n);
         auto inner = [&](auto& V) {
             using T = std::remove_pointer_t<decltype(V.r)>;
@@ -393,6 +396,8 @@ void free_batch(Batch* B) {
     drop_graph(B);
     if (B->pool) cudaFree(B->pool);
     B->pool = nullptr;
+    if (B->stage) cudaFreeHost(B->stage);
+    B->stage = nullptr;
     for (auto& e : B->ev) {
         if (e) cudaEventDestroy(e);
         e = nullptr;
@@ -526,6 +531,16 @@ int acs_batch_create(int32_t count, const acs_instance* members, const acs_setti
         std::vector<double>().swap(M.c);
         std::vector<int>().swap(M.soc_off);
     }
+    // pinned memory for one member's results, at most 4 MB; without it acs_batch_get
+    // copies to the caller's arrays directly
+    for (const Member& M : B->mem)
+        B->stage_bytes = std::max(B->stage_bytes, (size_t)(reinterpret_cast<const char*>(M.X.w + M.m) -
+                                                           reinterpret_cast<const char*>(M.x)));
+    B->stage_bytes = std::min(B->stage_bytes, (size_t)4 << 20);
+    if (cudaMallocHost(&B->stage, sizeof(Control) + B->stage_bytes) != cudaSuccess) {
+        B->stage = nullptr;
+        cudaGetLastError();
+    }
     const int rc = set_mapping(B, map0);
     if (rc != ACS_SOLVED) return fail(rc, -1);
     *out = reinterpret_cast<acs_batch*>(B);
@@ -579,20 +594,45 @@ int acs_batch_get(acs_batch* h, int32_t i, double* x, double* y, double* s, int3
     if (!B || i < 0 || i >= B->count) return ACS_ERR_ARG;
     if (cudaSetDevice(B->device) != cudaSuccess) return ACS_ERR_CUDA;
     const acs::Member& M = B->mem[i];
-    acs::Control C;
     cudaStream_t st = B->stream;
-    std::vector<double> w;
+    // the control block, and x, z and w (neighbours in the pool) in one copy, through
+    // pinned memory: each copy to pageable memory waits for the device (four of
+    // them took 45 us for a member of 500 rows).  A member whose results
+    // are larger than the stage is copied straight to the caller's arrays.
+    acs::Control local;
+    acs::Control& C = B->stage ? *reinterpret_cast<acs::Control*>(B->stage) : local;
+    const char* xs = B->stage + sizeof(acs::Control);
+    const char* dx = reinterpret_cast<const char*>(M.x);
+    const size_t span = (size_t)(reinterpret_cast<const char*>(M.X.w + M.m) - dx);
+    const bool staged = B->stage && span <= B->stage_bytes;
+    const double* w = nullptr;
+    std::vector<double> wtmp;
     if (cudaMemcpyAsync(&C, B->d_ctl + i, sizeof(C), cudaMemcpyDeviceToHost, st) != cudaSuccess) return ACS_ERR_CUDA;
-    if (x && cudaMemcpyAsync(x, M.x, sizeof(double) * M.n, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return ACS_ERR_CUDA;
-    if (s && cudaMemcpyAsync(s, M.z, sizeof(double) * M.n, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return ACS_ERR_CUDA;
-    if (y) {
-        w.resize(M.m);
-        if (cudaMemcpyAsync(w.data(), M.X.w, sizeof(double) * M.m, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (staged && (x || s || y)) {
+        if (cudaMemcpyAsync(B->stage + sizeof(acs::Control), dx, span, cudaMemcpyDeviceToHost, st) != cudaSuccess)
             return ACS_ERR_CUDA;
+        w = reinterpret_cast<const double*>(xs + (reinterpret_cast<const char*>(M.X.w) - dx));
+    } else if (!staged) {
+        if (x && cudaMemcpyAsync(x, M.x, sizeof(double) * M.n, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            return ACS_ERR_CUDA;
+        if (s && cudaMemcpyAsync(s, M.z, sizeof(double) * M.n, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            return ACS_ERR_CUDA;
+        if (y) {
+            try {
+                wtmp.resize(M.m);
+            } catch (...) {
+                return ACS_ERR_OOM;
+            }
+            if (cudaMemcpyAsync(wtmp.data(), M.X.w, sizeof(double) * M.m, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+                return ACS_ERR_CUDA;
+            w = wtmp.data();
+        }
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return ACS_ERR_CUDA;
+    if (staged) {
+        if (x) memcpy(x, xs, sizeof(double) * M.n);
+        if (s) memcpy(s, xs + (reinterpret_cast<const char*>(M.z) - dx), sizeof(double) * M.n);
+    }
     if (y) {
         const std::vector<int>& perm = B->mats[M.mat].H.perm;
         for (int r = 0; r < M.m; ++r) y[perm[r]] = w[r] / B->set.mu;
