@@ -203,7 +203,9 @@ inline unsigned short to_bf16(double v) {
 // assembly adds m^2 n / 2 multiply-adds, and the factor is 1.0 instead,
 // m^2 / n CG iterations (measured: one factorisation takes 109 ms at m = 2320,
 // n = 2900 against 60 us a CG iteration, 1.73 s at m = 8000, n = 1e4 against
-// 0.35 ms).
+// 0.35 ms).  These are the costs of an earlier factorisation, since made several
+// times faster; the rule stays as it is, because where a solve changes over
+// decides which iterates it takes.
 inline long long switch_budget(const acs_settings& set, int m, long long nnz, bool full_rows = false) {
     const double k = full_rows ? 1.0 : 0.3;
     const double f = k * (double)m * (double)m * (double)m / (double)(nnz > 0 ? nnz : 1);

@@ -106,7 +106,7 @@ __device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (
     // every lane of a warp runs the same number of rounds (its rows past m are empty)
     for (unsigned i0 = (t & ~31) / kLanes; i0 < (unsigned)P.m; i0 += nt / kLanes) {
         const unsigned i = i0 + (t & 31) / kLanes;
-        int k = 0, e = 0;
+        unsigned k = 0, e = 0;                           // k may pass e by a round: no overflow at 2^31
         double yi = 0.0;
         if (i < (unsigned)P.m) {
             k = P.rp[i] + l;
