@@ -19,10 +19,9 @@
 // matrix (18 us of HBM), one random read of x, two FP64 operations (32 us of a
 // pipe that does two multiply-adds per clock per SM) and one atomic add in L2.
 // Eight lanes a row make the matrix reads coalesced and keep short rows from
-// idling a warp.  A small problem is latency only, and runs as one kernel on one
-// thread-block cluster instead of four launches.  Measured: n = 1e6 476 ->
-// 160 us, n = 500 28 -> 16 us a call (before: a thread a row, and one thread
-// adding up the 1024 block partials).
+// idling a warp; the last block of the second kernel combines the partials.
+// Measured: n = 1e6 475 -> 155 us, n = 500 30 -> 18 us a call (before: a
+// thread a row, and a fourth kernel in which one thread added up the partials).
 
 #include <math.h>
 #include <mutex>
@@ -37,8 +36,6 @@ constexpr int kVals = 8;                       // partials per block
 constexpr int kThreadsNA = 1024;
 constexpr int kLanes = 8;                      // lanes a row of A, or a cone, is spread over
 constexpr int kHead = 2;                       // doubles before A'y: the counter of finished blocks
-constexpr int kSmallCtas = 8;                  // the one-cluster kernel (a portable cluster size)
-constexpr int kSmallThreads = 512;
 
 __device__ __align__(256) double g_noalloc_scratch[kHead + kMaxN + kMaxBlocks * kVals];
 
@@ -53,12 +50,12 @@ struct Args {
     unsigned* done;
 };
 
-// Block-wide sums of NV <= 16 values; the first NV threads write them to out.
+// Block-wide sums of NV <= 8 values; the first NV threads write them to out.
 // Inside a warp a lane gives half of its values away at each of the first steps,
 // so that eight values take nine additions a lane (the FP64 pipe is slow).
 template <int NV>
 __device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* out) {
-    constexpr int NP = NV <= 4 ? 4 : NV <= 8 ? 8 : 16;
+    constexpr int NP = NV <= 4 ? 4 : 8;
     __shared__ double sh[32][NP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     double a[NP];
@@ -76,7 +73,6 @@ __device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* o
     }
 #pragma unroll
     for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
-    __syncthreads();                                     // sh may still be read from an earlier call
     if ((lane & (32 / NP - 1)) == 0) sh[warp][lane / (32 / NP)] = a[0];
     __syncthreads();
     if (warp == 0) {
@@ -97,9 +93,8 @@ __device__ __forceinline__ double lanes_sum(double x) {
     return x;
 }
 
-// Rows of A, kLanes lanes a row: kDot: v += {||Ax - b||^2, b'y, ||b||^2};
-// kScatter: y_i A_ij into aty[j].  t, nt: this thread and the number of threads.
-template <bool kDot, bool kScatter>
+// Rows of A, kLanes lanes a row: v += {||Ax - b||^2, b'y, ||b||^2}; y_i A_ij into
+// aty[j].  t, nt: this thread and the number of threads.
 __device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (&v)[3]) {
     const int l = t % kLanes;
     constexpr int U = 4;
@@ -124,15 +119,14 @@ __device__ __forceinline__ void rows_part(const Args& P, int t, int nt, double (
                 a[u] = in ? __ldcs(P.av + k + u * kLanes) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) xj[u] = kDot && j[u] >= 0 ? P.x[j[u]] : 0.0;
+            for (int u = 0; u < U; ++u) xj[u] = j[u] >= 0 ? P.x[j[u]] : 0.0;
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (j[u] >= 0) {
-                    if (kDot) s = fma(a[u], xj[u], s);
-                    if (kScatter) atomicAdd(P.aty + j[u], a[u] * yi);
+                    s = fma(a[u], xj[u], s);
+                    atomicAdd(P.aty + j[u], a[u] * yi);
                 }
         }
-        if (!kDot) continue;
         s = lanes_sum(s);
         if (l == 0 && i < (unsigned)P.m) {
             const double bi = P.b[i], d = s - bi;
@@ -151,16 +145,12 @@ __device__ __forceinline__ double soc_dist2_na(double v1, double t) {
 }
 
 // Coordinates and cones (kLanes lanes a cone): v += {||A'y + z - c||^2, c'x,
-// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}; kRest: all but the first.
-template <bool kDual, bool kRest>
+// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}.
 __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (&v)[7]) {
     for (int j = t; j < P.n; j += nt) {
         const double xj = P.x[j], zj = P.z[j], cj = P.c[j];
-        if (kDual) {
-            const double d = __ldcg(P.aty + j) + zj - cj;
-            v[0] += d * d;
-        }
-        if (!kRest) continue;
+        const double d = __ldcg(P.aty + j) + zj - cj;
+        v[0] += d * d;
         v[6] += cj * cj;
         v[1] += cj * xj;
         const double xx = xj * xj, zz = zj * zj;
@@ -171,7 +161,6 @@ __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (
             if (zj < 0.0) v[5] += zz;
         }
     }
-    if (!kRest) return;
     const int l = t % kLanes;
     for (unsigned q0 = (t & ~31) / kLanes; q0 < (unsigned)P.n_soc; q0 += nt / kLanes) {
         const unsigned q = q0 + (t & 31) / kLanes;
@@ -243,14 +232,14 @@ __device__ __forceinline__ void finish_part(int nb_rows, int nb_cols, const doub
 
 __global__ void __launch_bounds__(kThreadsNA) rows_kernel(const Args P) {
     double v[3] = {0.0, 0.0, 0.0};
-    rows_part<true, true>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    rows_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
     block_sum_store<3>(v, P.prow + blockIdx.x * kVals);
 }
 
 // The block that ends last combines all partials.
 __global__ void __launch_bounds__(kThreadsNA) cols_kernel(const Args P, int nb_rows) {
     double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    cols_part<true, true>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
+    cols_part(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, v);
     block_sum_store<7>(v, P.pcol + blockIdx.x * kVals);
     if (threadIdx.x >= 32) return;
     __threadfence();
@@ -260,54 +249,6 @@ __global__ void __launch_bounds__(kThreadsNA) cols_kernel(const Args P, int nb_r
     if (!__shfl_sync(0xffffffffu, last, 0)) return;
     __threadfence();
     finish_part(nb_rows, (int)gridDim.x, P.prow, P.pcol, P.out);
-}
-
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// A small problem: the whole computation on one cluster, in the fewest steps one
-// after the other: everything that does not need A'y comes first, together with
-// clearing it, then the scatter, then r_d; ten sums a CTA go to CTA 0 through
-// distributed shared memory.
-__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads) small_kernel(const Args P) {
-    __shared__ double sums[10], all[kSmallCtas][10];
-    const int t = blockIdx.x * kSmallThreads + threadIdx.x;
-    constexpr int nt = kSmallCtas * kSmallThreads;
-    for (int j = t; j < P.n; j += nt) P.aty[j] = 0.0;
-    double v[3] = {0.0, 0.0, 0.0}, w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    rows_part<true, false>(P, t, nt, v);
-    cols_part<false, true>(P, t, nt, w);
-    cluster_barrier();
-    rows_part<false, true>(P, t, nt, v);
-    cluster_barrier();
-    cols_part<true, false>(P, t, nt, w);
-    const double both[10] = {v[0], v[1], v[2], w[0], w[1], w[2], w[3], w[4], w[5], w[6]};
-    block_sum_store<10>(both, sums);
-    if (threadIdx.x < 32) {
-        __syncwarp();
-        if (threadIdx.x < 10) {
-            unsigned remote;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
-                         : "=r"(remote)
-                         : "r"((unsigned)__cvta_generic_to_shared(&all[blockIdx.x][threadIdx.x])));
-            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(sums[threadIdx.x]) : "memory");
-        }
-    }
-    cluster_barrier();
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        double s[10];
-#pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            s[k] = lane < kSmallCtas ? all[lane][k] : 0.0;
-#pragma unroll
-            for (int o = kSmallCtas / 2; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
-            s[k] = __shfl_sync(0xffffffffu, s[k], 0);
-        }
-        write_residuals(s, P.out);
-    }
 }
 
 // Device address of the scratch array in the current device's context,
@@ -345,26 +286,23 @@ extern "C" int acs_kkt_residuals_noalloc(int32_t m, int32_t n, const int32_t* ro
            scratch + kHead + kMaxN, scratch + kHead + kMaxN + (kMaxBlocks / 2) * kVals, residuals,
            reinterpret_cast<unsigned*>(scratch)};
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // One cluster while even a full matrix is little work for its eight SMs (the
-    // number of nonzeros is on the device): m n <= 2^19 is at most 2^16
-    // multiply-adds a product on each, 16 us of FP64 pipe for both, against about
-    // 12 us of launches saved; a sparse problem of that size is latency only.
-    if ((long long)m * n <= (1LL << 19)) {
-        small_kernel<<<kSmallCtas, kSmallThreads, 0, st>>>(P);
-        return cudaGetLastError() == cudaSuccess ? ACS_SOLVED : ACS_ERR_CUDA;
-    }
-    // block counts in 64-bit arithmetic; at most two blocks of 1024 threads on
-    // each of 152 SMs, and never more than the scratch has partials for
+    // Blocks of 1024 threads, at most two on each of 152 SMs and never more than the
+    // scratch has partials for; where 304 blocks of 256 hold everything at once, those:
+    // the sums at a block's end take the FP64 pipe for each of its warps in turn.
+    // Measured, 256 / 1024 threads: m = 1000, n = 600 19 / 26 us, m = 2000, n = 5000
+    // 20 / 31.
     const long long most = 304 < kMaxBlocks / 2 ? 304 : kMaxBlocks / 2;
-    const long long rows_need = ((long long)m * kLanes + kThreadsNA - 1) / kThreadsNA;
-    const long long cols_need = ((long long)n + kThreadsNA - 1) / kThreadsNA;
-    const long long soc_need = ((long long)n_soc * kLanes + kThreadsNA - 1) / kThreadsNA;
+    const long long lanes_rows = (long long)m * kLanes;
+    const int t_rows = lanes_rows <= 256 * most ? 256 : kThreadsNA, t_cols = n <= 256 * most ? 256 : kThreadsNA;
+    const long long rows_need = (lanes_rows + t_rows - 1) / t_rows;
+    const long long cols_need = ((long long)n + t_cols - 1) / t_cols;
+    const long long soc_need = ((long long)n_soc * kLanes + t_cols - 1) / t_cols;
     const long long wide = cols_need > soc_need ? cols_need : soc_need;
     const int nb_rows = (int)(rows_need < most ? rows_need : most);
     const int nb_cols = (int)(wide < most ? wide : most);
     if (cudaMemsetAsync(scratch, 0, sizeof(double) * ((size_t)n + kHead), st) != cudaSuccess) return ACS_ERR_CUDA;
-    rows_kernel<<<nb_rows, kThreadsNA, 0, st>>>(P);
-    cols_kernel<<<nb_cols, kThreadsNA, 0, st>>>(P, nb_rows);
+    rows_kernel<<<nb_rows, t_rows, 0, st>>>(P);
+    cols_kernel<<<nb_cols, t_cols, 0, st>>>(P, nb_rows);
     if (cudaGetLastError() != cudaSuccess) return ACS_ERR_CUDA;
     return ACS_SOLVED;
 }
