@@ -43,6 +43,7 @@ std::mutex g_setup_mutex;
 
 struct Args {
     int m, n, n_orth, n_soc;
+    bool soc_short;                                // the mean cone has at most kLanes entries after its first
     const int *rp, *ci;
     const double *av, *b, *c, *x, *y, *z;
     const int* soc_off;
@@ -144,8 +145,8 @@ __device__ __forceinline__ double soc_dist2_na(double v1, double t) {
     return 2.0 * d * d;
 }
 
-// Coordinates and cones (kLanes lanes a cone): v += {||A'y + z - c||^2, c'x,
-// ||x||^2, ||z||^2, dist(x,K)^2, dist(z,K)^2, ||c||^2}.
+// Coordinates and cones: v += {||A'y + z - c||^2, c'x, ||x||^2, ||z||^2,
+// dist(x,K)^2, dist(z,K)^2, ||c||^2}.
 __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (&v)[7]) {
     for (int j = t; j < P.n; j += nt) {
         const double xj = P.x[j], zj = P.z[j], cj = P.c[j];
@@ -161,11 +162,59 @@ __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (
             if (zj < 0.0) v[5] += zz;
         }
     }
-    const int l = t % kLanes;
-    for (unsigned q0 = (t & ~31) / kLanes; q0 < (unsigned)P.n_soc; q0 += nt / kLanes) {
-        const unsigned q = q0 + (t & 31) / kLanes;
+    if (P.n_soc == 0) return;
+    // kLanes lanes a cone.  A root and a distance take the warp's FP64 instructions
+    // whether 2 or 32 lanes need them, so warps are numbered across the blocks
+    // first, and short cones (kLanes a group at a time) leave one cone to each lane
+    // before the roots.  Measured, cones' share of a call: n = 600, 300 cones
+    // of 2, 12 -> 4 us; n = 1e6, 5e5 cones of 2, 304 -> 53 us (before: eight lanes to
+    // every cone, warps in order).
+    const int lane = t & 31, l = lane % kLanes, g0 = lane - l;
+    const unsigned n_soc = (unsigned)P.n_soc, w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, nw = nt >> 5;
+    if (P.soc_short) {
+        for (unsigned q0 = w * 32; q0 < n_soc; q0 += nw * 32) {
+            const unsigned q = q0 + lane;
+            int a = 0, e = 0;
+            if (q < n_soc) {
+                a = P.soc_off[q];
+                e = P.soc_off[q + 1];
+            }
+            double sx[kLanes], sz[kLanes];
+#pragma unroll
+            for (int r = 0; r < kLanes; ++r) {           // the cone of lane g0 + r
+                const int j = __shfl_sync(0xffffffffu, a, g0 + r) + 1 + l, er = __shfl_sync(0xffffffffu, e, g0 + r);
+                const double xj = j < er ? P.x[j] : 0.0, zj = j < er ? P.z[j] : 0.0;
+                sx[r] = xj * xj;
+                sz[r] = zj * zj;
+                for (int i = j + kLanes; i < er; i += kLanes) {
+                    sx[r] = fma(P.x[i], P.x[i], sx[r]);
+                    sz[r] = fma(P.z[i], P.z[i], sz[r]);
+                }
+            }
+            int o = kLanes / 2;
+#pragma unroll
+            for (int c = kLanes; c > 1; c >>= 1, o >>= 1) {   // lane l keeps the sum of cone l
+                const bool up = (l & o) != 0;
+#pragma unroll
+                for (int i = 0; i < c / 2; ++i) {
+                    const double gx = up ? sx[i] : sx[i + c / 2], kx = up ? sx[i + c / 2] : sx[i];
+                    const double gz = up ? sz[i] : sz[i + c / 2], kz = up ? sz[i + c / 2] : sz[i];
+                    sx[i] = kx + __shfl_xor_sync(0xffffffffu, gx, o);
+                    sz[i] = kz + __shfl_xor_sync(0xffffffffu, gz, o);
+                }
+            }
+            if (q < n_soc) {
+                v[4] += soc_dist2_na(P.x[a], sqrt(sx[0]));
+                v[5] += soc_dist2_na(P.z[a], sqrt(sz[0]));
+            }
+        }
+        return;
+    }
+    constexpr unsigned per = 32 / kLanes;
+    for (unsigned q0 = w * per; q0 < n_soc; q0 += nw * per) {
+        const unsigned q = q0 + lane / kLanes;
         int a = 0, e = 0;
-        if (q < (unsigned)P.n_soc) {
+        if (q < n_soc) {
             a = P.soc_off[q];
             e = P.soc_off[q + 1];
         }
@@ -177,9 +226,8 @@ __device__ __forceinline__ void cols_part(const Args& P, int t, int nt, double (
         }
         sx = lanes_sum(sx);
         sz = lanes_sum(sz);
-        // lane 0 takes x, lane 1 z
-        if (q < (unsigned)P.n_soc && l < 2) {
-            const double d = l == 0 ? soc_dist2_na(P.x[a], sqrt(sx)) : soc_dist2_na(P.z[a], sqrt(sz));
+        if (q < n_soc && l < 2) {                        // lane 0 takes x, lane 1 z
+            const double d = soc_dist2_na(l == 0 ? P.x[a] : P.z[a], sqrt(l == 0 ? sx : sz));
             if (l == 0) v[4] += d;
             else v[5] += d;
         }
@@ -282,7 +330,8 @@ extern "C" int acs_kkt_residuals_noalloc(int32_t m, int32_t n, const int32_t* ro
     int err = ACS_SOLVED;
     double* scratch = scratch_for_current_device(&err);
     if (!scratch) return err;
-    Args P{m, n, n_orthant, n_soc, row_ptr, col, val, b, c, x, y, z, soc_offsets, scratch + kHead,
+    const bool soc_short = (long long)n - n_orthant <= (long long)n_soc * (kLanes + 1);
+    Args P{m, n, n_orthant, n_soc, soc_short, row_ptr, col, val, b, c, x, y, z, soc_offsets, scratch + kHead,
            scratch + kHead + kMaxN, scratch + kHead + kMaxN + (kMaxBlocks / 2) * kVals, residuals,
            reinterpret_cast<unsigned*>(scratch)};
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -292,11 +341,12 @@ extern "C" int acs_kkt_residuals_noalloc(int32_t m, int32_t n, const int32_t* ro
     // Measured, 256 / 1024 threads: m = 1000, n = 600 19 / 26 us, m = 2000, n = 5000
     // 20 / 31.
     const long long most = 304 < kMaxBlocks / 2 ? 304 : kMaxBlocks / 2;
+    const long long soc_block = soc_short ? 128 : 128 / kLanes;   // cones of four warps
+    const long long soc_need = (n_soc + soc_block - 1) / soc_block;
     const long long lanes_rows = (long long)m * kLanes;
     const int t_rows = lanes_rows <= 256 * most ? 256 : kThreadsNA, t_cols = n <= 256 * most ? 256 : kThreadsNA;
     const long long rows_need = (lanes_rows + t_rows - 1) / t_rows;
     const long long cols_need = ((long long)n + t_cols - 1) / t_cols;
-    const long long soc_need = ((long long)n_soc * kLanes + t_cols - 1) / t_cols;
     const long long wide = cols_need > soc_need ? cols_need : soc_need;
     const int nb_rows = (int)(rows_need < most ? rows_need : most);
     const int nb_cols = (int)(wide < most ? wide : most);

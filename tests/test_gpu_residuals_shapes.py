@@ -1,9 +1,11 @@
-"""The allocation-free residuals of tall and wide problems against the oracle's
-residual function.
+"""The allocation-free residuals of tall, wide and many-coned problems: against the
+oracle's residual function, and with short cones no dearer than their entries.
 
 Tolerance: as for the residuals' other tests, every output is a quotient of sums of
 at most n + nnz positive terms or of their roots, each off by at most its number of
 terms times eps; the two objectives by that times the sum of their magnitudes.
+Times: the smallest of several, as the ratio of two calls, bounded by about one and a
+half times what it should be.
 """
 import numpy as np
 import pytest
@@ -41,6 +43,18 @@ class Case:
                                             torch.cuda.current_stream().cuda_stream)
         assert rc == capi.SOLVED
 
+    def us(self):
+        best = np.inf
+        for _ in range(6):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            for _ in range(10):
+                self.call()
+            t1.record()
+            t1.synchronize()
+            best = min(best, t0.elapsed_time(t1) * 100.0)
+        return best
+
 
 @pytest.mark.parametrize("m,n,per_row", [(1, 524_288, 524_288), (3, 170_000, 170_000), (50_000, 10, 3),
                                          (524_288, 1, 1), (2048, 256, 10), (2049, 256, 10), (64, 16_384, 10),
@@ -56,6 +70,20 @@ def test_wide_with_cones(m, n):
     _check(Case(m, n, 10, [3] * (n // 3)))
 
 
+# cones of a mean length up to 9 are added up eight to a group of eight lanes, longer ones one to a group
+CONES = {"one": [7], "seven": [2, 3, 8, 9, 10, 5, 4], "eight": [9] * 8, "thirty-three": [3] * 33,
+         "a long one among short ones": [2] * 40 + [150] + [3] * 40, "of 10": [10] * 31, "of 64": [64] * 5,
+         "many": [2] * 400}
+
+
+@pytest.mark.parametrize("cones", sorted(CONES))
+@pytest.mark.parametrize("m", [40, 2600])
+@pytest.mark.parametrize("n_orth", [0, 13])
+def test_cones(cones, m, n_orth):
+    n = n_orth + sum(CONES[cones])
+    _check(Case(m, n, min(n, 4), CONES[cones]))
+
+
 def _check(P):
     ref = kkt.residuals(P.A, P.b, P.c, P.x, P.y, P.z, P.n_orth, P.dims)
     terms = 4 * (P.n + P.m + P.A.nnz)
@@ -67,3 +95,8 @@ def _check(P):
         for v, want, mag in ((got[4], ref["obj_p"], np.abs(P.c * P.x).sum()),
                              (got[5], ref["obj_d"], np.abs(P.b * P.y).sum())):
             assert abs(v - want) <= terms * EPS * mag
+
+
+def test_short_cones_cost_little():
+    """5e5 cones of 2 beside 1e7 nonzeros."""
+    assert Case(200_000, 1_000_000, 50, [2] * 500_000).us() <= 2.0 * Case(200_000, 1_000_000, 50, []).us()
