@@ -351,8 +351,10 @@ __device__ __forceinline__ bool gather_slots(const double* part, unsigned long l
 }
 
 // Barrier of all threads of the cluster; what any of them wrote before it is
-// visible to all after it.
+// visible to all after it.  barrier.cluster counts a warp when it arrives, so its lanes
+// have to arrive together; warp 0 comes here from code that only some of them run.
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
