@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <new>
 #include <atomic>
+#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -68,6 +69,7 @@ struct Batch {
     std::vector<Control> ctl_host;
     char* stage = nullptr;            // pinned: a member's control block and results on their way out
     size_t stage_bytes = 0;           //   (bytes of the results' part)
+    std::mutex stage_lock;            // one acs_batch_get at a time uses it
 };
 
 namespace {
@@ -598,7 +600,10 @@ int acs_batch_get(acs_batch* h, int32_t i, double* x, double* y, double* s, int3
     // the control block, and x, z and w (neighbours in the pool) in one copy, through
     // pinned memory: each copy to pageable memory waits for the device (four of
     // them took 45 us for a member of 500 rows).  A member whose results
-    // are larger than the stage is copied straight to the caller's arrays.
+    // are larger than the stage is copied straight to the caller's arrays.  The
+    // stage is the batch's, so calls from several threads take turns.
+    std::unique_lock<std::mutex> lock(B->stage_lock, std::defer_lock);
+    if (B->stage) lock.lock();
     acs::Control local;
     acs::Control& C = B->stage ? *reinterpret_cast<acs::Control*>(B->stage) : local;
     const char* xs = B->stage + sizeof(acs::Control);
