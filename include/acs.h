@@ -302,7 +302,9 @@ const char* acs_status_string(int status);
  * FP64 A' passes, conditionings, FP64 iterations} of the last solve (the
  * benchmark's algorithmic-byte model counts matrix passes with these).
  * acs_problem_info: out8 = {m, n, nnz, stored entries of A and of A' after padding,
- * CTAs of the FP32 launch, CTAs of the FP64 launch, threads per CTA}. */
+ * CTAs of the FP32 launch, CTAs of the FP64 launch, threads per CTA}.  A small problem
+ * with the cached operator has one launch, a thread-block cluster: the last two are its
+ * 8 or 16 CTAs of 512 threads (else 1024). */
 int acs_debug_counters(acs_problem* p, long long* out6);
 /* Device time (ms) of the last persistent iteration launch, from CUDA events
  * recorded on the handle's stream around that launch; waits for it.  After an

@@ -842,7 +842,9 @@ int acs_problem_info(acs_problem* h, int32_t* out8) {
     out8[0] = P->m; out8[1] = P->n; out8[2] = P->nnz;
     out8[3] = (int32_t)std::min<long long>(P->padded_A, INT32_MAX);
     out8[4] = (int32_t)std::min<long long>(P->padded_AT, INT32_MAX);
-    out8[5] = P->grid32; out8[6] = P->grid64; out8[7] = acs::kThreads;
+    out8[5] = P->grid32;
+    out8[6] = P->small_ctas > 0 ? P->small_ctas : P->grid64;
+    out8[7] = P->small_ctas > 0 ? acs::kSmallThreads : acs::kThreads;
     return ACS_SOLVED;
 }
 

@@ -14,6 +14,7 @@
 namespace acs {
 
 constexpr int kThreads = 1024;          // threads per CTA of the persistent kernel
+constexpr int kSmallThreads = 512;      // ... of the one-cluster launch of small problems (acs_small.cu)
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRed = 8;              // doubles reduced per grid reduction
 // A CTA's partials, (value, generation) pairs: two sets, used by barriers of

@@ -16,8 +16,6 @@
 namespace acs {
 namespace {
 
-constexpr int kSmallThreads = 512;
-
 __global__ void __launch_bounds__(kSmallThreads, 1) small_iter_kernel(const __grid_constant__ IterParams<double> P) {
     if (ld_volatile_int(&P.ctl->status) != ST_RUNNING) return;
     team_set(blockIdx.x, gridDim.x, &P.ctl->bar_count64, P.partials, P.dM, P.dX, 1);
