@@ -34,6 +34,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) small_iter_kernel(const __gr
 // 28.1 (0.58), m = 400 25.9 (1.4) / 31.3 (1.0), m = 512 27.6 (2.1) / 31.2
 // (1.25: at 100 iterations a factorisation the grid is ahead), m = 700 37.7 /
 // 32.5; dense SOCP m = 200 36.5 / 48.8, m = 296 53.9 / 56.7, m = 400 69 / 61.
+// Coordinates and cones cost too: at two rounds of them the grid is ahead for sparse
+// rows (m = 200 with 2 entries a column: n = 10000 27.8 / 25.7, n = 20000 34.3 / 27.2,
+// n = 40000 50.7 / 30.8; two full rows the other way, n = 20000 88 / 114), and a wider
+// problem is left to it.
 int small_cluster(const Problem* P) {
     if (P->dense != 1) return 0;
     const double work = (double)P->m * P->m + (double)P->padded_A + (double)P->padded_AT;
@@ -46,6 +50,7 @@ int small_cluster(const Problem* P) {
         return 0;
     }
     for (int c = kMaxCluster; c >= 8; c /= 2) {
+        if (P->n > 2 * c * kSmallThreads) return 0;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(c);
         cfg.blockDim = dim3(kSmallThreads);
