@@ -320,16 +320,17 @@ int acs_last_polish_ms(acs_problem* p, double* ms);
  * factorisation, cached-operator correction, and for the column-blocked
  * passes the three phases that add up their partial sums: t = O^2 A'u of
  * the CG, the projection residual and the update of the FP32 outer passes,
- * then the cached operator's assembly of M and its inverse factor (the
- * factorisation entry covers the Cholesky steps).  n >= 18.  Returns the
+ * then the cached operator's assembly of M and the transposition of its inverse
+ * factor (the factorisation entry covers factor and inverse, one sweep).  n >= 18.  Returns the
  * number of phases written or an error. */
 int acs_debug_phase_times(acs_problem* p, double* ms, long long* count, int32_t n);
 /* Mean time (ns) of one grid-wide reduce-and-barrier of the persistent
- * kernel's launch shape, over n back-to-back barriers. */
+ * kernel's grid launch, over n back-to-back barriers.  (A small problem with
+ * the cached operator runs as one cluster, with the hardware's barrier.) */
 int acs_debug_barrier_ns(acs_problem* p, int32_t n, double* ns);
 int acs_problem_info(acs_problem* p, int32_t* out8);
 /* Test of the failure path of the persistent kernel's grid barrier: one
- * grid-wide barrier of the solve's launch shape at which one CTA never
+ * grid-wide barrier of the grid launch at which one CTA never
  * arrives.  The others' bounded waits (2 s) run out; they record
  * ACS_ERR_DEVICE_TIMEOUT and leave the kernel, which returns normally (no
  * trap; the context and the handle stay usable).  Returns the recorded

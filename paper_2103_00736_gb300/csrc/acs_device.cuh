@@ -21,14 +21,6 @@ __device__ __forceinline__ unsigned long long gtimer() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ int ld_volatile_int(const int* p) { return *(volatile const int*)p; }
 
 // Grid-wide reduction and barrier.
@@ -49,10 +41,13 @@ __device__ __forceinline__ int ld_volatile_int(const int* p) { return *(volatile
 // 13.7 -> 8.7 us, a KKT check of a 1000 x 5000 LP 34 -> 21 us (before: every
 // CTA read the partials after the counter had arrived, and every thread
 // computed the scalars).
-// All waits are bounded
+// All waits through memory are bounded
 // (kBarrierTimeoutNs): on expiry, or when another CTA has recorded an error,
 // the wait records ACS_ERR_DEVICE_TIMEOUT and grid_sync returns false in
-// every thread; the caller then leaves the kernel.
+// every thread; the caller then leaves the kernel.  A team that is one cluster
+// waits in the hardware's barrier.cluster, which has no limit and needs none as
+// long as all CTAs leave the loop at the same barrier.  They do: the FP64 loop
+// without bulk copies ends only on values that every CTA holds alike.
 constexpr int kMaxGrid = 256;   // CTAs of a persistent launch (one per SM)
 constexpr int kMaxCluster = 16; // CTAs of a launch that is one cluster
 
@@ -210,7 +205,7 @@ __device__ __forceinline__ bool is_nonzero(double x) {   // without the FP64 pip
 // one value per warp (warps with nothing but zeros skip their sums).  op: 0 =
 // sum, 1 = max.
 template <int NV>
-__device__ __forceinline__ void block_partials(const double (&v)[NV], const int (&op)[NV], double* /*unused*/) {
+__device__ __forceinline__ void block_partials(const double (&v)[NV], const int (&op)[NV]) {
     SyncShared& S = sync_smem();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned mask = 0u;
@@ -384,8 +379,8 @@ __device__ __forceinline__ void st_cluster(double* var, int rank, double v) {
 //
 // A team that is one cluster uses the hardware's cluster barrier (which counts
 // threads that have not exited, so it cannot wait for a CTA that has left) and
-// exchanges partials through distributed shared memory.  A team of one CTA
-// needs neither.  The caller follows with a CTA barrier.
+// exchanges partials through distributed shared memory; it reads the error word at
+// reducing barriers only.  A team of one CTA needs neither.  The caller follows with a CTA barrier.
 static __device__ __noinline__ void grid_reduce(int* err) {
     SyncShared& S = sync_smem();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -516,7 +511,7 @@ __device__ __forceinline__ bool grid_sync(int* err) {
 
 // Values reduced at the last grid_sync.
 template <int NV>
-__device__ void grid_combine(const double* /*unused*/, const int (&)[NV], double (&out)[NV]) {
+__device__ void grid_combine(double (&out)[NV]) {
     SyncShared& S = sync_smem();
 #pragma unroll
     for (int k = 0; k < NV; ++k) out[k] = S.out[k];
@@ -1177,13 +1172,6 @@ __device__ __forceinline__ void for_cones(const P_& P, Body body) {
     }
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T x) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
 // Is iteration l in the schedule L (Algorithm 2 step 4, without the {1})?
 template <typename T>
 __device__ __forceinline__ bool in_schedule(const IterParams<T>& P, int l) {
@@ -1233,7 +1221,7 @@ __device__ __noinline__ void phase_cond_o(const IterParams<T>& P) {
     });
     const double v[3] = {vmax, vneg, good};
     const int op[3] = {1, 1, 0};
-    block_partials<3>(v, op, P.partials);
+    block_partials<3>(v, op);
 }
 
 // Exponent range (CondRange) of step 11 over the finite positive o.  An o of 0, inf or
@@ -1293,7 +1281,7 @@ __device__ __noinline__ void phase_btilde(const IterParams<T>& P) {
     sell_rows2(P.A, g1, g2, epi);
     const double v[1] = {bad};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // Start of the projection solve: w <- w + theta (w - w_prev) and, since
@@ -1392,7 +1380,7 @@ __device__ __noinline__ void phase_rhs(const IterParams<T>& P) {
     sell_rows<double>(P.A, gather, epi);
     const double v[1] = {gam};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // FP32 outer products on the L2-gather layout (a segment that need only reach
@@ -1407,7 +1395,7 @@ __device__ __noinline__ void phase_rhs_f32(const IterParams<T>& P) {
     sell_rows<float>(P.A, gather, epi);
     const double v[1] = {gam};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // FP32 outer passes: the product A g of the projection residual as a
@@ -1423,7 +1411,7 @@ __device__ __noinline__ void phase_rhs_comb(const IterParams<T>& P) {
     cb_combine(P.Acb, &P.ctl->err, [&](int i, float sum) { rhs_epi(P, i, (double)sum, gam); });
     const double v[1] = {gam};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // CG, first half of M u: t = O^2 (A' u) over the rows of A'.
@@ -1448,7 +1436,7 @@ __device__ __noinline__ void phase_cg_A(const IterParams<T>& P) {
     sell_rows<T>(P.A, gather, epi);
     const double v[1] = {delta};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // Column-blocked CG, first half of M u: the partial sums of A'u ...
@@ -1469,7 +1457,7 @@ __device__ __noinline__ void phase_cg_tcomb(const IterParams<T>& P) {
     });
     const double v[1] = {delta};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 // Column-blocked CG, second half: the partial sums of A t (= M u), combined
 // in the vector step.
@@ -1538,7 +1526,7 @@ __device__ __noinline__ void phase_cg_vec(const IterParams<T>& P) {
         for (int i = global_tid(); i < P.m; i += global_threads()) step(i, V.au[i]);
     const double v[1] = {gam};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // q = O (A' w) over the rows of A' (FP64); with update: s <- (s + p)/2 -
@@ -1601,12 +1589,12 @@ __device__ __forceinline__ void update_epi(const IterParams<T>& P, int j, double
 // Partials of the update: ||s_new - s||^2, ||s_new||^2 and, for a
 // time-sliced solve, the CTAs that have seen the deadline pass (one clock
 // read per CTA, summed, so every CTA of the team takes the same decision).
-__device__ __forceinline__ void update_partials(double ds2, double ss2, bool update, double* partials) {
+__device__ __forceinline__ void update_partials(double ds2, double ss2) {
     const unsigned long long dl = sync_smem().deadline;
-    const double over = (update && dl != 0ull && threadIdx.x == 0 && gtimer() > dl) ? 1.0 : 0.0;
+    const double over = (dl != 0ull && threadIdx.x == 0 && gtimer() > dl) ? 1.0 : 0.0;
     const double v[3] = {ds2, ss2, over};
     const int op[3] = {0, 0, 0};
-    block_partials<3>(v, op, partials);
+    block_partials<3>(v, op);
 }
 
 // q = A_hat' w and g = O (p + q) alone: the start of a solve in a new scaling, and
@@ -1631,7 +1619,7 @@ __device__ __noinline__ void phase_update_form(const IterParams<T>& P, bool want
     auto gather = [w](int i) { return w[i]; };
     auto epi = [&](int j, double sum) { update_epi(P, j, sum, true, want_xz, ds2, ss2, fuse_abs, kAdmm); };
     sell_rows<double>(P.AT, gather, epi);
-    update_partials(ds2, ss2, true, P.partials);
+    update_partials(ds2, ss2);
 }
 template <typename T>
 __device__ __forceinline__ void phase_update(const IterParams<T>& P, bool update, bool want_xz, bool fuse_abs = false) {
@@ -1648,7 +1636,7 @@ __device__ __noinline__ void phase_update_f32(const IterParams<T>& P, bool want_
     auto gather = [w](int i) { return (float)w[i]; };
     auto epi = [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs, P.admm != 0); };
     sell_rows<float>(P.AT, gather, epi);
-    update_partials(ds2, ss2, true, P.partials);
+    update_partials(ds2, ss2);
 }
 
 // FP32 outer passes: A'w as a column-blocked FP32 pass (w rounded to FP32 as
@@ -1663,7 +1651,7 @@ __device__ __noinline__ void phase_update_comb(const IterParams<T>& P, bool want
     double ds2 = 0.0, ss2 = 0.0;
     cb_combine(P.ATcb, &P.ctl->err,
                [&](int j, float sum) { update_epi(P, j, (double)sum, true, want_xz, ds2, ss2, fuse_abs, P.admm != 0); });
-    update_partials(ds2, ss2, true, P.partials);
+    update_partials(ds2, ss2);
 }
 
 // ADMM form, Lorentz cones: abs_K of the reflection a kept in p by
@@ -1702,7 +1690,7 @@ __device__ __noinline__ void phase_admm_soc(const IterParams<T>& P, bool want_xz
     });
     const double v[2] = {ds2, ss2};
     const int op[2] = {0, 0};
-    block_partials<2>(v, op, P.partials);
+    block_partials<2>(v, op);
 }
 
 // FP64 residual partials: ||Ax - b||^2, ||A'y + z - c||^2 (y = w/mu), c'x, b'y,
@@ -1773,7 +1761,7 @@ __device__ __noinline__ void phase_kkt(const IterParams<T>& P) {
     });
     const double v[8] = {rp, rd, cx, by, dx, dz, xx, zz};
     const int op[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    block_partials<8>(v, op, P.partials);
+    block_partials<8>(v, op);
 }
 
 // ---------------------------------------------------------------------------
@@ -2217,8 +2205,9 @@ __device__ __noinline__ bool dense_factor_step(double* M, double* X, int m, int 
 // by O_j^2), the next slab's entries loaded while one is multiplied.  FP64
 // throughout; the FP64 pipe bounds it (a slab is 4 us), so the tiles are kept
 // small: n = 200, m = 160 has 15 of them.  Measured: m = 160, n = 200 on 16 CTAs
-// 65 us (233 on the grid before), m = 800, n = 1000 1.14 -> 0.90 ms (before: 64
-// x 64 tiles, 1024-thread CTAs only, without the prefetch).
+// 65 us (233 on the grid before), m = 800, n = 1000 1.14 -> 0.90 ms, m = 8000, n =
+// 10000 612 -> 630 ms (before: 64 x 64 tiles, 1024-thread CTAs only, without the
+// prefetch; with 200 tiles to a CTA the larger ones load half as much).
 template <int R, typename T>
 __device__ __forceinline__ void dense_syrk(const IterParams<T>& P) {
     DenseShared& S = dense_smem();
@@ -2285,7 +2274,7 @@ __device__ __noinline__ void phase_dense_assemble(const IterParams<T>& P) {
 // dM <- X' (upper triangle, row-major), 32 x 32 tiles through shared memory.
 static __device__ __noinline__ void dense_transpose(const double* X, double* Mt, int m) {
     DenseShared& S = dense_smem();
-    double(*tile)[kTile + 1] = reinterpret_cast<double(*)[kTile + 1]>(&S);   // 8.4 KB of its 13
+    double(*tile)[kTile + 1] = reinterpret_cast<double(*)[kTile + 1]>(&S);   // 8.4 KB of its 24
     const int nt = (m + kTile - 1) / kTile;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (unsigned u = team_rank(); u < (unsigned)nt * (unsigned)(nt + 1) / 2u; u += team_size()) {
@@ -2408,7 +2397,7 @@ static __device__ __noinline__ void phase_polish_init(const IterParams<double>& 
     for (int i = global_tid(); i < P.m; i += global_threads()) P.X.w[i] = 0.0;
     const double v[1] = {nb};
     const int op[1] = {0};
-    block_partials<1>(v, op, P.partials);
+    block_partials<1>(v, op);
 }
 
 // b_tilde = b and J^{-1} = 1 / diag(A_B A_B') (1 on rows without an entry in B).
@@ -2517,7 +2506,7 @@ __device__ __noinline__ void phase_polish_rhs(const IterParams<T>& P) {
     sell_rows2(P.A, g1, g2, epi);
     const double v[2] = {gam, fl};
     const int op[2] = {0, 0};
-    block_partials<2>(v, op, P.partials);
+    block_partials<2>(v, op);
 }
 
 // M w = b_tilde - A g by FP64 refinement rounds (FP64 residual, Jacobi-PCG
@@ -2629,8 +2618,7 @@ static __device__ __noinline__ void polish_loop(const IterParams<double>& P, con
         phase_polish_init(P, fp32 ? P32.V.O2 : nullptr);
         if (!grid_sync(&P.ctl->err)) break;
         {
-            const int op[1] = {0};
-            grid_combine<1>(P.partials, op, nb);
+            grid_combine<1>(nb);
         }
         if (fp32) phase_polish_jacobi(P32);
         else phase_polish_jacobi(P);
@@ -2663,8 +2651,7 @@ static __device__ __noinline__ void polish_loop(const IterParams<double>& P, con
         phase_kkt(Q);
         if (!grid_sync(&P.ctl->err)) break;
         double r8[8];
-        const int op[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        grid_combine<8>(P.partials, op, r8);
+        grid_combine<8>(r8);
         if (owner) {
             out.res[0] = sqrt(r8[0]) / (1.0 + P.bnorm);
             out.res[1] = sqrt(r8[1]) / (1.0 + P.cnorm);

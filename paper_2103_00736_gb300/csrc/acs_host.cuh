@@ -151,10 +151,10 @@ inline int validate(int32_t m, int32_t n, const int64_t* row_ptr, const int32_t*
     return ACS_SOLVED;
 }
 
-// Lanes that share one Lorentz cone: enough that the longest cone takes no more
-// than 64 rounds (a lone long cone must not serialise a few lanes), and no fewer
-// than 4 (a 32-byte sector of FP64 values), else eight entries a lane of the
-// mean cone.
+// Lanes that share one Lorentz cone: no fewer than 4 (a 32-byte sector of FP64
+// values) and up to 32, enough for no more than 64 rounds of the longest cone (a
+// lone long cone must not serialise a few lanes; above 2048 entries 32 lanes take
+// more rounds) and for twelve entries a lane of the mean cone.
 inline int soc_lanes(int n_soc, const int* off) {
     if (n_soc <= 0) return 32;
     int longest = 0;

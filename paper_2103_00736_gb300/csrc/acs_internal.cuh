@@ -41,8 +41,8 @@ enum Phase : int {
     PH_CG_TCOMB,     // column-blocked CG: t = O^2 (A'u) from the partial sums, and u'Mu
     PH_RHS_COMB,     // FP32 outer passes: the projection residual from the partial sums
     PH_UPD_COMB,     // FP32 outer passes: q = A_hat' w from the partial sums and the update
-    PH_DENSE_ASSEMBLE,   // cached operator: M = A O^2 A' (PH_DENSE_FACTOR: its Cholesky steps)
-    PH_DENSE_INVERSE,    // cached operator: L^{-1}
+    PH_DENSE_ASSEMBLE,   // cached operator: M = A O^2 A' (PH_DENSE_FACTOR: M = L L' and L^{-1} in one sweep)
+    PH_DENSE_INVERSE,    // cached operator: the transposition of L^{-1}
     PH_COUNT
 };
 

@@ -53,10 +53,10 @@ barrier_probe_kernel(Control* ctl, unsigned* flags, double* partials, int n, dou
     for (int i = 0; i < n; ++i) {
         const double v[1] = {1.0};
         const int op[1] = {0};
-        block_partials<1>(v, op, partials);
+        block_partials<1>(v, op);
         if (!grid_sync(&ctl->err)) break;
         double r[1];
-        grid_combine<1>(partials, op, r);
+        grid_combine<1>(r);
         acc += r[0];
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {

@@ -3,11 +3,10 @@
 // A problem of a few hundred constraints with the cached projection operator
 // does 1e4 to 1e6 FP64 multiply-adds an iteration in four phases; on the whole
 // grid its time is the grid barriers (2 us each, 4 with a reduction) and the
-// instructions that 152 x 32 mostly idle warps spend around them (spills of the
-// 64-register build included: a third of the instructions).  On one cluster the
-// barrier is the hardware's, partials travel through distributed shared memory,
-// and 512 threads a CTA have 128 registers each, so the phases are compiled into
-// the loop.  The FP64 pipe then sets the limit: 2 multiply-adds per clock per SM
+// instructions that 152 x 32 mostly idle warps spend around them (16 % of them
+// spills of the 64-register build).  On one cluster the barrier is the hardware's,
+// partials travel through distributed shared memory, and 512 threads a CTA have
+// 128 registers each, so nothing spills.  The FP64 pipe then sets the limit: 2 multiply-adds per clock per SM
 // on 16 SMs instead of 152, hence the size rule in small_cluster().
 #include <cuda_runtime.h>
 
